@@ -59,7 +59,7 @@ def peaks():
 def kernel_hash() -> str:
     h = hashlib.sha256()
     for f in ("ed_apply.cu", "ed_apply_impl.cuh", "ed_device.cuh", "ed_internal.h", "ed_cache.cu", "ed_cache.cuh",
-              "ed_cache_lanes.cu"):
+              "ed_cache_pass.cu"):
         h.update(open(os.path.join(ROOT, "paper_2210_03511_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -626,7 +626,7 @@ def main():
         b_alg, kernel = b_free, "hx_kernel"
     else:
         b_alg = stored_bytes(D, gathers, s_x)
-        kernel = "cache_pass_lanes" if store["lanes_per_row"] > 1 else "cache_pass_kernel"
+        kernel = "cache_pass_split" if store["lanes_per_row"] > 1 else "cache_pass_kernel"
     achieved = b_alg / t_launch / 1e9
     traffic, ncu_ctx = profiled_traffic(args.workload, dtype, kernel)
     launches_per_step = 1 if args.matrix_free else store["segments"]

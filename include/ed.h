@@ -326,7 +326,10 @@ ed_status ed_apply(const ed_hamiltonian* h, ed_dtype dtype, const void* x, void*
  * structure would need more than max_bytes, nothing is kept and
  * ED_ERR_NOMEM is returned (ed_apply stays matrix-free).  Also
  * ED_ERR_TABLE_TOO_LARGE when more than 256 distinct coefficients occur,
- * ED_ERR_ARG for more than 255 flip terms.  Synchronous on `stream`.
+ * ED_ERR_ARG for more than 255 flip terms.  The build takes scratch from the
+ * same allocator (8 bytes per flip term for a chunk of rows, up to about 3 GB;
+ * 64 MB when the allocator has no room for that), released on return.
+ * Synchronous on `stream`.
  * A second call replaces the stored structure. */
 ed_status ed_hamiltonian_store(ed_hamiltonian* h, ed_dtype dtype, int32_t seg_log2, size_t max_bytes,
                                ed_stream stream, size_t* bytes);
@@ -340,7 +343,7 @@ ed_status ed_hamiltonian_store(ed_hamiltonian* h, ed_dtype dtype, int32_t seg_lo
  * (ed_hamiltonian_store_set_lanes), and the fastest pair is kept (the
  * structure built again if it was not the last one tried).  Fewer, larger
  * segments save the per-row work of each pass; smaller ones keep the gathered
- * part of x in L2; several lanes per row balance long rows across a warp.
+ * part of x in L2; several lanes per row spread long rows over more warps.
  * *seg_log2 (if non-NULL) receives the chosen log2 segment size, *bytes the
  * structure's size (ed_hamiltonian_store_schedule reports both choices).
  * Errors as ed_hamiltonian_store.  Synchronous. */
@@ -350,10 +353,9 @@ ed_status ed_hamiltonian_store_autotune(ed_hamiltonian* h, ed_dtype dtype, size_
 /* ed_hamiltonian_store_set_lanes -- work split of the stored pass for ONE
  * vector (several vectors always take one lane per row): lanes_per_row = 1
  * (the default after every ed_hamiltonian_store: one lane per row, a row's
- * elements summed in stored order, one warp per 32 rows) or 2, 4, 8 (groups of
- * that many consecutive lanes share a row; element k goes to lane k mod L of
- * the group and a butterfly of warp shuffles combines the lanes' sums; a warp
- * still owns 32 rows and takes them in L rounds).  Results differ from one
+ * elements summed in stored order, one warp per 32 rows) or 2, 4, 8 (that many
+ * warps share 32 rows: the q-th takes the q-th part of every row's elements,
+ * and the parts' sums are added in order).  Results differ from one
  * lane per row only by summation order (the bit-identity with the
  * matrix-free kernel holds for one lane per row).  ED_ERR_ARG for other
  * values or without a stored structure. */

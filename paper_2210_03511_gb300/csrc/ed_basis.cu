@@ -207,28 +207,17 @@ __global__ void scan_tile_apply(const uint32_t* in, uint64_t n, const uint64_t* 
         }
 }
 
-// Exclusive scan of n u32 values into u64 offsets (device), total to the host.
-ed_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, uint64_t* total, const Alloc& A,
+uint64_t scan_scratch_words(uint64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
+
+// Exclusive scan of n u32 values into u64 offsets (device).
+ed_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, uint64_t* tiles, uint64_t* total,
                              cudaStream_t s) {
-    const uint64_t n_tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-    const size_t bytes = (size_t)(n_tiles + 2) * 8;
-    uint64_t* tiles = (uint64_t*)A.get(bytes, s);
-    if (!tiles) return fail(ED_ERR_NOMEM, "scan scratch");
-    uint64_t* d_total = tiles + n_tiles + 1;
-    ed_status st = ED_OK;
-    if (n_tiles) {
-        scan_tile_sums<<<(unsigned)n_tiles, 256, 0, s>>>(in, n, tiles);
-        scan_tiles_serial<<<1, 1024, 0, s>>>(tiles, n_tiles, d_total);
-        scan_tile_apply<<<(unsigned)n_tiles, 256, 0, s>>>(in, n, tiles, out);
-    } else {
-        cudaMemsetAsync(d_total, 0, 8, s);
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(total, d_total, 8, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) st = cuda_fail(e, "exclusive scan");
-    A.put(tiles, bytes, s);
-    return st;
+    const uint64_t n_tiles = scan_scratch_words(n);
+    scan_tile_sums<<<(unsigned)n_tiles, 256, 0, s>>>(in, n, tiles);
+    scan_tiles_serial<<<1, 1024, 0, s>>>(tiles, n_tiles, total);
+    scan_tile_apply<<<(unsigned)n_tiles, 256, 0, s>>>(in, n, tiles, out);
+    ED_CUDA(cudaGetLastError());
+    return ED_OK;
 }
 
 // ---------------------------------------------------------------- Limits
@@ -859,8 +848,7 @@ ed_status basis_build_device(ed_basis* b, cudaStream_t s) {
     Seg* d_segs = (Seg*)sc.get(segs.size() * sizeof(Seg));
     uint32_t* d_counts = (uint32_t*)sc.get(chunks * 4);
     uint64_t* d_offs = (uint64_t*)sc.get(chunks * 8);
-    const uint64_t n_tiles = (chunks + SCAN_TILE - 1) / SCAN_TILE;
-    uint64_t* d_tiles = (uint64_t*)sc.get(n_tiles * 8 + 8);
+    uint64_t* d_tiles = (uint64_t*)sc.get(scan_scratch_words(chunks) * 8);
     uint64_t* d_total = (uint64_t*)sc.get(8);
     if (!d_segs || !d_counts || !d_offs || !d_tiles || !d_total) return fail(ED_ERR_NOMEM, "enumeration scratch");
     ED_CUDA(cudaMemcpyAsync(d_segs, segs.data(), segs.size() * sizeof(Seg), cudaMemcpyHostToDevice, s));
@@ -879,10 +867,8 @@ ed_status basis_build_device(ed_basis* b, cudaStream_t s) {
     a.counts = d_counts;
     st = run_enum(b, a, 0, sms, s);
     if (st != ED_OK) return st;
-    scan_tile_sums<<<(unsigned)n_tiles, 256, 0, s>>>(d_counts, chunks, d_tiles);
-    scan_tiles_serial<<<1, 1024, 0, s>>>(d_tiles, n_tiles, d_total);
-    scan_tile_apply<<<(unsigned)n_tiles, 256, 0, s>>>(d_counts, chunks, d_tiles, d_offs);
-    ED_CUDA(cudaGetLastError());
+    st = exclusive_scan_u32(d_counts, chunks, d_offs, d_tiles, d_total, s);
+    if (st != ED_OK) return st;
     uint64_t D = 0;
     ED_CUDA(cudaMemcpyAsync(&D, d_total, 8, cudaMemcpyDeviceToHost, s));
     ED_CUDA(cudaStreamSynchronize(s));

@@ -140,18 +140,20 @@ struct ed_basis {
 };
 
 namespace ed {
-// Stored structure of H (csrc/ed_cache.cu): per column segment b, entry
-// counts per row, per-slice offsets and the entries (code << 24 | column
-// offset), the per-row Ising part, and the coefficient table of the codes.
+// Stored structure of H (layout: csrc/ed_cache.cu): per column segment the
+// rows' entry counts, per-slice offsets, the entries (code |
+// column offset) by chunks of slices, the per-row Ising part, and the
+// coefficient tables of the codes.
 struct HCache {
     bool valid = false;
     int seg_bits = 0, nb = 0, n_code = 0, sms = 0, off_bits = 24;
     bool axis_d = false, axis_f = false;  // complex codes all real or purely imaginary (FP64 / FP32 table)
     int n_re = 0;                         // codes below n_re have real coefficients
     int lanes = 1;                        // lanes per row of the one-vector pass (1, 2, 4, 8)
-    int64_t ns = 0;                 // slices of 32 rows
-    DevBuf counts, boff, ent, diag, ctab, ctr;
-    std::vector<uint64_t> bbase;    // [nb+1] first entry of each segment
+    int chunk_shift = 0;                  // slice >> chunk_shift = chunk
+    int64_t ns = 0;                       // slices of 32 rows
+    DevBuf counts, boff, diag, ctab, base;  // base: the chunks' entry addresses
+    std::vector<DevBuf> ent;              // entries of each chunk
     uint64_t n_ent = 0, n_skip = 0;
     size_t bytes = 0;
 };
@@ -206,17 +208,18 @@ HxArgs make_args(const ed_hamiltonian* h);
 // One sector's stored structure as the batched stored-structure kernel reads
 // it (one column segment; see csrc/ed_cache.cu).
 struct CacheSector {
-    const uint8_t* counts;     // [32 ns] entries per row
-    const uint32_t* boff;      // [ns] first entry of each slice
-    const uint32_t* ent;       // entries: (code << off_bits) | column
+    const uint8_t* counts;     // [32 ns] entries of each row
+    const uint32_t* boff;      // [ns] first entry of each slice in its chunk
+    const uint32_t* const* ent;  // entries of each chunk: (code << off_bits) | column
     const double* diag;        // [D] Ising part
     const uint16_t* stab;      // [D] |Stab sigma_i|
-    const uint8_t* ctab;       // coefficients: [256] double2, [256] double, [256] float2, [256] float
+    const uint8_t* ctab;       // coefficient tables (csrc/ed_cache.cuh)
     const uint8_t* sq;         // sqrt(k) then 1/sqrt(k), k = 0..G (double)
     const uint8_t* sqf;        // the same in float
     int64_t D, ns, slice0;     // rows, slices, first slice of the sector in the batch's slice list
     int G1;                    // G + 1
     uint32_t off_bits;
+    int64_t chunk_shift;
 };
 // One batched H.x launch (all sectors of a batch).
 struct BatchLaunch {
@@ -241,8 +244,8 @@ struct BatchLaunch {
     int64_t stored_slices;     // slices of 32 rows over all sectors
 };
 ed_status apply_batch_launch(const BatchLaunch& L, cudaStream_t s);
-// implemented in ed_cache.cu: the batched stored-structure H.x, and the
-// descriptor of one Hamiltonian's structure (false unless stored in one segment)
+// the batched stored-structure H.x (ed_cache_pass.cu), and the descriptor of
+// one Hamiltonian's structure (ed_cache.cu; false unless stored in one segment)
 ed_status cache_batch_launch(const BatchLaunch& L, cudaStream_t s);
 bool cache_sector_desc(const ed_hamiltonian* h, CacheSector& d);
 size_t hx_smem_bytes(const ed_hamiltonian* h, ed_dtype dt, bool ns_ok, int nvec, int blocks);
@@ -255,7 +258,9 @@ ed_status representatives_device(const ed_basis* b, const uint64_t* states, int6
                                  int32_t* nstab, uint8_t* compat, cudaStream_t s);
 ed_status representatives_static(const ed_sector* sector, const uint64_t* states, int64_t n, uint64_t* rep, int32_t* g,
                                  int32_t* nstab, uint8_t* compat, cudaStream_t s);
-ed_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, uint64_t* total, const Alloc& A,
+// exclusive scan of n values (n > 0) into out, the total to *total; tiles: scan_scratch_words(n) words of scratch (all device)
+uint64_t scan_scratch_words(uint64_t n);
+ed_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, uint64_t* tiles, uint64_t* total,
                              cudaStream_t s);
 // implemented in ed_apply.cu; uses the stored structure when there is one and use_cache is set
 ed_status apply_launch(const ed_hamiltonian* h, ed_dtype dt, const void* x, void* y, int nvec, cudaStream_t s,
