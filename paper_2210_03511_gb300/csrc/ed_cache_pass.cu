@@ -23,15 +23,20 @@ namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 
-// Resident blocks per SM of a pass launch (register budget 65536 / (256 x blocks)).
-constexpr int pass_blocks(int K, int NV) { return NV == 1 ? (K == 2 ? 5 : 6) : 2; }
+// Entries in flight per lane, and resident blocks per SM (register budget
+// 65536 / (256 x blocks)).  Four entries at 5 blocks (4 for complex FP64) beat
+// more warps with fewer entries in flight and fewer warps with eight: square36
+// FP64 13.5 ms against 14.3 (4 and 2 in the ragged rest, 6 blocks), 15.1 (2, 8
+// blocks) and 13.8 (8, 4 blocks); kagome36 complex FP32 14.2 against 16.2, 17.0
+// and 15.3; square32 FP64 0.334 against 0.344, 0.366 and 0.329.
+constexpr int AHEAD = 4;
+constexpr int pass_blocks(int K, int NV) { return NV == 1 ? (K == 2 ? 4 : 5) : 2; }
 
 // Walk entries [k0, k1) of every row of a slice in order (c: entries of this
 // lane's row; p: the slice's first entry; k0, k1 and p uniform over the warp).
-// get(w) loads x for entry word w, use(w, x) adds it.  U entries are in flight
-// per lane while all 32 rows have one; the ragged rest goes two at a time, the
-// places of the rows that still have an entry from ballots.
-template <int U, typename X, typename Get, typename Use>
+// get(w) loads x for entry word w, use(w, x) adds it.  Once a row of the slice
+// has ended, the places of the others' entries come from ballots.
+template <typename X, typename Get, typename Use>
 __device__ __forceinline__ void walk(uint32_t c, const uint32_t* p, uint32_t k0, uint32_t k1, int lane, Get&& get,
                                      Use&& use) {
     const uint32_t cmin = __reduce_min_sync(FULL, c);
@@ -40,30 +45,35 @@ __device__ __forceinline__ void walk(uint32_t c, const uint32_t* p, uint32_t k0,
     if (k0) q += __reduce_add_sync(FULL, min(c, k0));
     const uint32_t kf = min(cmin, k1);
     uint32_t k = k0;
-    for (; k + U <= kf; k += U, q += 32 * U) {
-        uint32_t w[U];
-        X xv[U];
+    for (; k + AHEAD <= kf; k += AHEAD, q += 32 * AHEAD) {
+        uint32_t w[AHEAD];
+        X xv[AHEAD];
 #pragma unroll
-        for (int u = 0; u < U; ++u) w[u] = __ldg(q + 32 * u + lane);
+        for (int u = 0; u < AHEAD; ++u) w[u] = __ldg(q + 32 * u + lane);
 #pragma unroll
-        for (int u = 0; u < U; ++u) xv[u] = get(w[u]);
+        for (int u = 0; u < AHEAD; ++u) xv[u] = get(w[u]);
 #pragma unroll
-        for (int u = 0; u < U; ++u) use(w[u], xv[u]);
+        for (int u = 0; u < AHEAD; ++u) use(w[u], xv[u]);
     }
     const unsigned lt = (1u << lane) - 1u;
-    for (; k < k1; k += 2) {
-        const bool h0 = c > k, h1 = c > k + 1 && k + 1 < k1;
-        const unsigned m0 = __ballot_sync(FULL, h0), m1 = __ballot_sync(FULL, h1);
-        const int n0 = __popc(m0);
-        uint32_t w0 = 0, w1 = 0;
-        if (h0) w0 = __ldg(q + __popc(m0 & lt));
-        if (h1) w1 = __ldg(q + n0 + __popc(m1 & lt));
-        X x0, x1;
-        if (h0) x0 = get(w0);
-        if (h1) x1 = get(w1);
-        if (h0) use(w0, x0);
-        if (h1) use(w1, x1);
-        q += n0 + __popc(m1);
+    for (; k < k1; k += AHEAD) {
+        uint32_t w[AHEAD];
+        X xv[AHEAD];
+        bool has[AHEAD];
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+            has[u] = c > k + u && k + u < k1;
+            const unsigned m = __ballot_sync(FULL, has[u]);
+            w[u] = 0;
+            if (has[u]) w[u] = __ldg(q + __popc(m & lt));
+            q += __popc(m);
+        }
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u)
+            if (has[u]) xv[u] = get(w[u]);
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u)
+            if (has[u]) use(w[u], xv[u]);
     }
 }
 
@@ -81,8 +91,7 @@ __device__ __forceinline__ void accumulate(R& re, R& im, const CT& cf, bool imag
         re += cf.x * (imag ? x.y : x.x);
         im += cf.y * (imag ? x.x : x.y);
     } else {
-        re += cf.x * x.x - cf.y * x.y;
-        im += cf.x * x.y + cf.y * x.x;
+        cmadd(re, im, cf.x, cf.y, x);
     }
 }
 
@@ -178,14 +187,14 @@ __global__ void __launch_bounds__(BLOCK, pass_blocks(K, NV)) cache_pass_kernel(C
             }
         }
         if constexpr (NV == 1) {
-            walk<4, T>(
+            walk<T>(
                 c, ent, 0u, 255u, lane, [&](uint32_t w) { return xs[w & om]; },
                 [&](uint32_t w, const T& xj) {
                     const uint32_t cd = w >> ob;
                     accumulate<K, AX>(re[0], im[0], ctab[cd], cd >= n_re, xj);
                 });
         } else {
-            walk<2, char>(
+            walk<char>(
                 c, ent, 0u, 255u, lane, [&](uint32_t) { return (char)0; },
                 [&](uint32_t w, char) {
                     const uint32_t cd = w >> ob;
@@ -238,7 +247,7 @@ __global__ void __launch_bounds__(BLOCK, pass_blocks(K, 1)) cache_pass_split(Cac
             Ahead a;
             a.load(p, sl, lane);
             const uint32_t n = __reduce_max_sync(FULL, a.c);
-            walk<4, T>(
+            walk<T>(
                 a.c, a.base + a.bo, n * q / L, n * (q + 1) / L, lane, [&](uint32_t w) { return xs[w & om]; },
                 [&](uint32_t w, const T& xj) { accumulate<K, false>(re, im, ctab[w >> ob], false, xj); });
         }
@@ -277,7 +286,7 @@ __global__ void __launch_bounds__(BLOCK, pass_blocks(K, 1)) cache_pass_split(Cac
 // advance by x_step_elems per device-side step (block Lanczos graphs);
 // sectors with active[s] == 0 are skipped.
 template <int K, int NV>
-__global__ void __launch_bounds__(BLOCK, NV == 1 ? 6 : 2)
+__global__ void __launch_bounds__(BLOCK, pass_blocks(K, NV))
     cache_batch_kernel(const CacheSector* __restrict__ sec, int n_sec, int64_t n_slices,
                        const int64_t* __restrict__ row_off, const void* xv, void* yv, int nvec,
                        const int* __restrict__ x_step, int64_t x_step_elems, const int* __restrict__ active) {
@@ -316,11 +325,11 @@ __global__ void __launch_bounds__(BLOCK, NV == 1 ? 6 : 2)
 #pragma unroll
         for (int v = 0; v < NV; ++v) re[v] = im[v] = 0;
         if constexpr (NV == 1) {
-            walk<4, T>(
+            walk<T>(
                 n, ent, 0u, 255u, lane, [&](uint32_t w) { return x[w & om]; },
                 [&](uint32_t w, const T& xj) { accumulate<K, false>(re[0], im[0], coef(w), false, xj); });
         } else {
-            walk<2, char>(
+            walk<char>(
                 n, ent, 0u, 255u, lane, [&](uint32_t) { return (char)0; },
                 [&](uint32_t w, char) {
                     const CT cf = coef(w);
@@ -396,9 +405,10 @@ ed_status cache_batch_launch(const BatchLaunch& L, cudaStream_t s) {
     ED_CUDA(cudaGetDevice(&dev));
     ED_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t blocks_needed = (L.stored_slices + (BLOCK / 32) - 1) / (BLOCK / 32);
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(blocks_needed, (int64_t)sms * 6));
     auto go = [&](auto ktag) -> ed_status {
         constexpr int K = decltype(ktag)::value;
+        const int64_t fit = (int64_t)sms * pass_blocks(K, L.nvec == 1 ? 1 : MAXV);
+        const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(blocks_needed, fit));
         if (L.nvec == 1)
             cache_batch_kernel<K, 1><<<grid, BLOCK, 0, s>>>(L.stored, L.n_sec, L.stored_slices, L.row_off, L.x, L.y,
                                                             L.nvec, L.x_step, L.x_step_elems, L.active);
