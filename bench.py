@@ -59,7 +59,7 @@ def peaks():
 def kernel_hash() -> str:
     h = hashlib.sha256()
     for f in ("ed_apply.cu", "ed_apply_impl.cuh", "ed_device.cuh", "ed_internal.h", "ed_cache.cu", "ed_cache.cuh",
-              "ed_cache_pass.cu"):
+              "ed_cache_pass.cu", "ed_cache_walk.cuh", "ed_cache_multi.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2210_03511_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 

@@ -33,15 +33,6 @@ template <> struct Val<1> { using T = float; using R = float; static constexpr b
 template <> struct Val<2> { using T = double2; using R = double; static constexpr bool cplx = true; };
 template <> struct Val<3> { using T = float2; using R = float; static constexpr bool cplx = true; };
 
-// (re, im) += (cr + i ci) x as four multiply-adds.  Written as
-// re += cr x.re - ci x.im the product difference is formed first and added
-// after: three FP64 instructions per part instead of two.
-template <typename R, typename T>
-__device__ __forceinline__ void cmadd(R& re, R& im, R cr, R ci, const T& x) {
-    re = fma(-ci, x.y, fma(cr, x.x, re));
-    im = fma(ci, x.x, fma(cr, x.y, im));
-}
-
 constexpr int MAXV = 8;
 constexpr int BLOCK = 256;        // threads per block
 constexpr int MAXW = 8;           // activity mask words per row (n_flip <= 256)
@@ -276,7 +267,8 @@ __device__ __forceinline__ void hx_body(const HxArgs& a, uint8_t* smem, int64_t 
                     for (int v = 0; v < NV; ++v)
                         if (v < nvec) {
                             const T xj = x[(int64_t)v * D + jx];
-                            cmadd(accr[v], acci[v], cr, ci, xj);
+                            accr[v] += cr * xj.x - ci * xj.y;
+                            acci[v] += cr * xj.y + ci * xj.x;
                         }
                 }
             }

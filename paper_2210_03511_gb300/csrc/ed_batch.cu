@@ -47,6 +47,7 @@ struct ed_batch {
     mutable std::vector<ed::CacheSector> stored_h;
     mutable ed::DevBuf d_stored;
     mutable int64_t stored_slices = 0;
+    mutable ed::StreamPool scratch;        // interleaved copies of several FP32 vectors
 };
 
 namespace ed {
@@ -800,7 +801,11 @@ ed_status ed_apply_batch(const ed_batch* B, ed_dtype dtype, const void* x, void*
     BatchLaunch L = make_launch(B, dtype, x, y, nvec);
     if (B->has_sun && !L.stored) return fail(ED_ERR_ARG, "a batch with SU(N) sectors needs every sector's stored structure");
     ED_CUDA(cudaMemsetAsync(B->d_counters.p, 0, 24, (cudaStream_t)stream));
-    return apply_batch_launch(L, (cudaStream_t)stream);
+    const size_t copy = L.stored ? cache_interleaved_bytes(dtype, nvec, B->total) : 0;
+    if (copy) L.xi = B->scratch.get(*B->alloc, B->hs[0]->basis->device, copy, (cudaStream_t)stream);
+    const ed_status st = apply_batch_launch(L, (cudaStream_t)stream);
+    if (L.xi) StreamPool::put(L.xi, (cudaStream_t)stream);
+    return st;
 }
 
 ed_status ed_batch_autotune(ed_batch* B, ed_dtype dtype, const void* x, void* y, int32_t nvec, ed_stream stream,
@@ -969,6 +974,8 @@ static ed_status block_lanczos(const ed_batch* B, const ed_block_lanczos_opts* o
     L.active = active;
     L.x_step = dk;
     L.x_step_elems = bs;
+    const size_t copy = L.stored ? cache_interleaved_bytes(o->dtype, b, tot) : 0;
+    if (copy) L.xi = get(copy);  // without it: one vector after another
     auto step = [&]() -> ed_status {
         ed_status st = apply_batch_launch(L, s);  // W = H V_k
         if (st != ED_OK) return st;

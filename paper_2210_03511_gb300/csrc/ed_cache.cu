@@ -697,22 +697,25 @@ ed_status cache_apply(const ed_hamiltonian* h, ed_dtype dt, const void* x, void*
     p.off_bits = (uint32_t)c.off_bits;
     p.n_re = (uint32_t)c.n_re;
     const int K = dt == ED_F64 ? 0 : dt == ED_F32 ? 1 : dt == ED_C128 ? 2 : 3;
+    const size_t copy = cache_interleaved_bytes(dt, nvec, b->dim);
+    if (copy) p.xi = h->scratch.get(b->alloc, b->device, copy, s);
     const bool f64 = K == 0 || K == 2;
-    // several warps per slice: the general tables
-    const bool ax = K >= 2 && !(nvec == 1 && c.lanes > 1) && (f64 ? c.axis_d : c.axis_f);
+    // several warps per slice, interleaved vectors: the general tables
+    const bool ax = K >= 2 && !p.xi && !(nvec == 1 && c.lanes > 1) && (f64 ? c.axis_d : c.axis_f);
     const uint8_t* ct = (const uint8_t*)c.ctab.p;
     p.ctab = ct + (f64 ? (ax ? CT_AXD : CT_D2) : (ax ? CT_AXF : CT_F2));
     p.isq = b->dt.blob + (f64 ? b->dt.off_sqrt + (size_t)(b->ht.G + 1) * 8 : b->dt.off_sqrtf + (size_t)(b->ht.G + 1) * 4);
-    for (int k = 0; k < c.nb; ++k) {
+    ed_status st = ED_OK;
+    for (int k = 0; k < c.nb && st == ED_OK; ++k) {
         p.counts = (const uint8_t*)c.counts.p + (size_t)k * c.ns * NSLICE;
         p.boff = (const uint32_t*)c.boff.p + (size_t)k * c.ns;
         p.xoff = (int64_t)k << c.seg_bits;
         p.mode = c.nb == 1 ? 0 : (k == 0 ? 1 : (k == c.nb - 1 ? 3 : 2));
         p.counters = k == 0 ? (unsigned long long*)h->d_counters.p : nullptr;
-        const ed_status st = launch_cache_pass(p, K, ax, c.lanes, c.sms, s);
-        if (st != ED_OK) return st;
+        st = launch_cache_pass(p, K, ax, c.lanes, c.sms, s);
     }
-    return ED_OK;
+    if (p.xi) StreamPool::put(p.xi, s);
+    return st;
 }
 
 }  // namespace ed

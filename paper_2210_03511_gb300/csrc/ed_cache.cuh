@@ -20,6 +20,7 @@ struct CachePass {
     const uint32_t* boff;       // [ns] first entry of each slice, relative to its chunk's entries
     const uint32_t* const* ent; // [chunks] entries of each chunk of slices
     const void* x;              // [nvec][D]
+    void* xi;                   // several FP32 vectors: room for their copy interleaved by row (filled at mode 0 and 1), or null
     void* y;                    // [nvec][D]
     const void* ctab;           // [256] complex coefficients of the value kind's precision
     const void* isq;            // [G+1] 1/sqrt(k) of the value kind's real type
@@ -34,8 +35,8 @@ struct CachePass {
     unsigned long long n_ent, n_skip;
 };
 
-// One segment's pass for p.nvec vectors of kind K, `lanes` warps per slice
-// (one vector).  ax: p.ctab is the axis-aligned table.
+// One segment's pass for p.nvec vectors of kind K, `lanes` warps per slice for
+// one vector.  ax: p.ctab is the axis-aligned table (never with p.xi).
 ed_status launch_cache_pass(const CachePass& p, int K, bool ax, int lanes, int sms, cudaStream_t s);
 
 }  // namespace ed

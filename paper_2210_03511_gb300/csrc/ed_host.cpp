@@ -58,6 +58,36 @@ void Alloc::put(void* p, size_t bytes, cudaStream_t s) const {
     else cudaFree(p);
 }
 
+void* StreamPool::get(const Alloc& A, int device, size_t bytes, cudaStream_t s) {
+    if (A.custom) return nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    std::lock_guard<std::mutex> l(mu);
+    if (!pool) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        uint64_t keep = KEEP;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            if (pool) cudaMemPoolDestroy(pool);
+            pool = nullptr;
+            return nullptr;
+        }
+    }
+    void* p = nullptr;
+    if (cudaMallocFromPoolAsync(&p, bytes, pool, s) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return p;
+}
+
 // ------------------------------------------------------------------ sector validation + Alg. 1
 static std::string elem_key(const int32_t* p, int N, uint8_t f) {
     std::string k((const char*)p, (size_t)N * sizeof(int32_t));

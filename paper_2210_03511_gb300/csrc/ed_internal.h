@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <mutex>
 #include <vector>
 
 #include "ed.h"
@@ -33,6 +34,23 @@ struct Alloc {
 struct DevBuf {
     void* p = nullptr;
     size_t bytes = 0;
+};
+
+// Device scratch of calls that are asynchronous on their stream: a
+// stream-ordered memory pool of its owner (a Hamiltonian, a batch), made on
+// first use and destroyed with the owner.  Calls on several streams or threads
+// each get memory of their own; up to KEEP bytes stay in the pool between
+// calls.  get returns null (the caller then does without) for a custom
+// allocator, on a capturing stream, and when the memory is not there.
+struct StreamPool {
+    static constexpr uint64_t KEEP = 256ull << 20;
+    std::mutex mu;
+    cudaMemPool_t pool = nullptr;
+    void* get(const Alloc& A, int device, size_t bytes, cudaStream_t s);
+    static void put(void* p, cudaStream_t s) { cudaFreeAsync(p, s); }
+    ~StreamPool() {
+        if (pool) cudaMemPoolDestroy(pool);
+    }
 };
 
 // ---------------------------------------------------------------- sublattice-coding tables (host)
@@ -177,6 +195,7 @@ struct ed_hamiltonian {
     int tuned_blocks[4][2] = {};        // resident H.x blocks per SM by dtype, nvec == 1 / > 1 (0: default)
     bool sun = false;                   // SU(N) exchange model: applied through its stored structure only
     ed::HCache cache;                   // stored structure, when built (ed_hamiltonian_store)
+    mutable ed::StreamPool scratch;     // interleaved copies of several FP32 vectors (stored H.x)
 };
 
 namespace ed {
@@ -242,11 +261,14 @@ struct BatchLaunch {
     const int* active;         // device [n_sec]: rows of sectors with 0 are skipped (null: all)
     const CacheSector* stored; // device [n_sec]: every sector's stored structure, or null (matrix-free)
     int64_t stored_slices;     // slices of 32 rows over all sectors
+    void* xi;                  // stored structures, several FP32 vectors: room for their interleaved copy, or null
 };
 ed_status apply_batch_launch(const BatchLaunch& L, cudaStream_t s);
 // the batched stored-structure H.x (ed_cache_pass.cu), and the descriptor of
 // one Hamiltonian's structure (ed_cache.cu; false unless stored in one segment)
 ed_status cache_batch_launch(const BatchLaunch& L, cudaStream_t s);
+// bytes of the interleaved copy of nvec vectors of `rows` rows (0: none is made)
+size_t cache_interleaved_bytes(ed_dtype dt, int nvec, int64_t rows);
 bool cache_sector_desc(const ed_hamiltonian* h, CacheSector& d);
 size_t hx_smem_bytes(const ed_hamiltonian* h, ed_dtype dt, bool ns_ok, int nvec, int blocks);
 int hx_default_blocks(const ed_hamiltonian* h, ed_dtype dt, bool ns_ok, int nvec);
