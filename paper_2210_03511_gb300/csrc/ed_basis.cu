@@ -220,6 +220,12 @@ ed_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, uint
     return ED_OK;
 }
 
+// first basis index of every segment
+__global__ void segment_starts(const Seg* segs, int n_segs, const uint64_t* chunk_off, uint64_t* start) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_segs; i += gridDim.x * blockDim.x)
+        start[i] = chunk_off[segs[i].chunk0];
+}
+
 // ---------------------------------------------------------------- Limits
 // Two-level Limits: for top-block value v, bucket b = next q_v bits;
 // key = base_v + b; limits[key] = first index with state >= (v, b).
@@ -885,15 +891,20 @@ ed_status basis_build_device(ed_basis* b, cudaStream_t s) {
     a.stab = (uint16_t*)b->stab.p;
     st = run_enum(b, a, 1, sms, s);
     if (st != ED_OK) return st;
-    // per-segment dimensions from the chunk offsets
-    std::vector<uint64_t> offs(chunks);
-    ED_CUDA(cudaMemcpyAsync(offs.data(), d_offs, chunks * 8, cudaMemcpyDeviceToHost, s));
+    // per-segment dimensions from the chunk offsets (gathered on the device: there are
+    // millions of chunks and a few thousand segments)
+    std::vector<uint64_t> first(segs.size());
+    uint64_t* d_first = (uint64_t*)sc.get(segs.size() * 8);
+    if (!d_first) return fail(ED_ERR_NOMEM, "enumeration scratch");
+    segment_starts<<<(unsigned)((segs.size() + 255) / 256), 256, 0, s>>>(d_segs, (int)segs.size(), d_offs, d_first);
+    ED_CUDA(cudaGetLastError());
+    ED_CUDA(cudaMemcpyAsync(first.data(), d_first, segs.size() * 8, cudaMemcpyDeviceToHost, s));
     ED_CUDA(cudaStreamSynchronize(s));
     std::vector<uint64_t> v_lo(S + 1, 0);
     {
         // v_lo[v] = first index with top block >= v
         std::vector<uint64_t> start(S, UINT64_MAX);
-        for (size_t i = 0; i < segs.size(); ++i) start[segs[i].v] = offs[segs[i].chunk0];
+        for (size_t i = 0; i < segs.size(); ++i) start[segs[i].v] = first[i];
         uint64_t next = D;
         v_lo[S] = D;
         for (int v = S - 1; v >= 0; --v) {

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "ed_internal.h"
 
 // Helpers are __host__ __device__ so the exact device logic can also run on the
@@ -243,16 +245,19 @@ ED_HD void find_rep(W s, const TabView<CHUNKED>& t, W& rep, int& gbest, int& nst
     compat = cp;
 }
 
-// find_rep for a compile-time number of blocks NS (2..4).  Substates, block
-// representatives and the best image so far (block by block) live in
-// registers.  Each candidate g reads its packed (source block, map id)
-// entries for all destination blocks with one 8-byte load and composes its
-// image from the most significant destination block down, stopping at the
-// first block that exceeds the best image (most candidates stop after one
-// lookup).  Same outputs as find_rep.
+// find_rep for a compile-time number of blocks NS (2..4).  Substates and block
+// representatives live in registers; a candidate g reads its packed (source
+// block, map id) entries for all destination blocks with one 8-byte load, looks
+// all its blocks up at once and compares whole images.  A warp runs this loop as
+// long as its lane with the most candidates (1.5 on average, 5 in the slowest of
+// 32 lanes), so the loop is kept short: no exit in the middle of an image, no
+// turn of its own for moving on to the next list, characters read only on a tie
+// (36-site kagome sector: @@).
+// Same outputs as find_rep.
 template <typename W, bool CHUNKED, int NS>
 ED_HD void find_rep_ns(W s, const TabView<CHUNKED>& t, W& rep, int& gbest, int& nstab, bool& compat) {
     static_assert(NS >= 2 && NS <= 4, "specialised for 2..4 blocks");
+    using I = typename std::conditional<(NS <= 3), uint32_t, uint64_t>::type;  // blocks 1.. of an image, m <= 16
     const int m = t.m;
     const int S = 1 << m;
     uint32_t sub[NS], r[NS];
@@ -263,65 +268,57 @@ ED_HD void find_rep_ns(W s, const TabView<CHUNKED>& t, W& rep, int& gbest, int& 
         r[X] = t.rep[X * S + sub[X]];
         minrep = r[X] < minrep ? r[X] : minrep;
     }
-    uint32_t bestb[NS];
-#pragma unroll
-    for (int Z = 0; Z < NS; ++Z) bestb[Z] = 0xFFFFFFFFu;
-    bestb[0] = minrep;
-    bool have = false;
-    int gb = 0, ns = 0;
-    bool cp = true;
-    uint32_t cls = 0;
-    // One flat loop over the concatenated Sym_Y lists of all blocks Y with
-    // Rep_Y = MinRep: a separate loop per Y would make a warp wait for the
-    // longest list of every Y in turn.
-    uint32_t ymask = 0;
+    uint32_t ymask = 0;  // blocks Y with Rep_Y = MinRep whose Sym_Y list is still to come
 #pragma unroll
     for (int Y = 0; Y < NS; ++Y) ymask |= (r[Y] == minrep ? 1u : 0u) << Y;
     uint32_t q = 0, q1 = 0;
-    while (true) {
-        if (q == q1) {
-            if (!ymask) break;
-            const int Y = ctz32(ymask);
-            ymask &= ymask - 1;
-            uint32_t sy = sub[0];
+    auto next_list = [&]() {
+        const int Y = ctz32(ymask);
+        ymask &= ymask - 1;
+        uint32_t sy = sub[0];
 #pragma unroll
-            for (int k = 1; k < NS; ++k) sy = (Y == k) ? sub[k] : sy;
-            q = t.sym_off[Y * (S + 1) + sy];
-            q1 = t.sym_off[Y * (S + 1) + sy + 1];
-            continue;
-        }
-        const int g = t.sym_ids[q++];
+        for (int k = 1; k < NS; ++k) sy = (Y == k) ? sub[k] : sy;
+        q = t.sym_off[Y * (S + 1) + sy];
+        q1 = t.sym_off[Y * (S + 1) + sy + 1];
+    };
+    auto image = [&](int g) -> I {
         const uint2 pk = *(const uint2*)(t.dl + (size_t)g * 4);
         const uint32_t ent[4] = {pk.x & 0xFFFFu, pk.x >> 16, pk.y & 0xFFFFu, pk.y >> 16};
-        uint32_t v[NS];
-        v[0] = minrep;
-        int state = have ? 0 : -1;  // 0: equal so far, -1: smaller, 1: larger
+        I img = 0;
 #pragma unroll
         for (int Z = 1; Z < NS; ++Z) {
-            if (state == 1) break;
             const uint32_t X = ent[Z] >> 12;
             uint32_t sx = sub[0];
 #pragma unroll
             for (int k = 1; k < NS; ++k) sx = (X == (uint32_t)k) ? sub[k] : sx;
-            v[Z] = sym_action<CHUNKED>(t, ent[Z] & 0xFFFu, sx);
-            if (state == 0) state = v[Z] > bestb[Z] ? 1 : (v[Z] < bestb[Z] ? -1 : 0);
+            img = (img << m) | (I)sym_action<CHUNKED>(t, ent[Z] & 0xFFFu, sx);
         }
-        if (state == 1) continue;
-        if (state == -1) {
-#pragma unroll
-            for (int Z = 1; Z < NS; ++Z) bestb[Z] = v[Z];
-            have = true;
-            gb = g; ns = 1; cls = t.chi_cls[g]; cp = true;
-        } else {
+        return img;
+    };
+    next_list();  // a list of a block that reaches MinRep is never empty
+    int g = t.sym_ids[q];
+    I best = image(g);
+    int ns = 1;
+    bool cp = true;
+    while (true) {
+        if (++q == q1) {
+            if (!ymask) break;
+            next_list();
+        }
+        const int c = t.sym_ids[q];
+        const I img = image(c);
+        if (img < best) {
+            best = img;
+            g = c;
+            ns = 1;
+            cp = true;
+        } else if (img == best) {
             ++ns;
-            cp = cp && (t.chi_cls[g] == cls);
+            cp = cp && t.chi_cls[c] == t.chi_cls[g];
         }
     }
-    W best = 0;
-#pragma unroll
-    for (int Z = 0; Z < NS; ++Z) best = (best << m) | (W)bestb[Z];
-    rep = best;
-    gbest = gb;
+    rep = ((W)minrep << ((NS - 1) * m)) | (W)best;
+    gbest = g;
     nstab = ns;
     compat = cp;
 }

@@ -8,7 +8,6 @@
 #include <algorithm>
 #include <map>
 #include <string>
-#include <unordered_map>
 #include <vector>
 
 #include "ed_internal.h"
@@ -89,10 +88,51 @@ void* StreamPool::get(const Alloc& A, int device, size_t bytes, cudaStream_t s) 
 }
 
 // ------------------------------------------------------------------ sector validation + Alg. 1
-static std::string elem_key(const int32_t* p, int N, uint8_t f) {
-    std::string k((const char*)p, (size_t)N * sizeof(int32_t));
-    k.push_back((char)f);
-    return k;
+// The group elements by their permutation and flip (open addressing): a sector
+// looks up |G|^2 products, so a lookup allocates nothing.
+class ElemIndex {
+    const HostTables& t;
+    std::vector<int> slot;
+    size_t mask;
+    static uint64_t hash(const int32_t* p, int N, uint8_t f) {
+        uint64_t h = 0xCBF29CE484222325ull ^ f;
+        for (int i = 0; i < N; ++i) h = (h ^ (uint64_t)p[i]) * 0x100000001B3ull;
+        return h ^ (h >> 29);
+    }
+    bool is(int g, const int32_t* p, uint8_t f) const {
+        return t.flip[g] == f && memcmp(&t.perm[(size_t)g * t.N], p, (size_t)t.N * sizeof(int32_t)) == 0;
+    }
+
+  public:
+    explicit ElemIndex(const HostTables& tables) : t(tables) {
+        size_t n = 4;
+        while (n < (size_t)t.G * 4) n *= 2;
+        slot.assign(n, -1);
+        mask = n - 1;
+    }
+    int find(const int32_t* p, uint8_t f) const {
+        for (size_t i = hash(p, t.N, f) & mask;; i = (i + 1) & mask) {
+            if (slot[i] < 0 || is(slot[i], p, f)) return slot[i];
+        }
+    }
+    // element g, unless an equal one is there (returned; -1 when added)
+    int add(int g) {
+        const int32_t* p = &t.perm[(size_t)g * t.N];
+        const int e = find(p, t.flip[g]);
+        if (e >= 0) return e;
+        size_t i = hash(p, t.N, t.flip[g]) & mask;
+        while (slot[i] >= 0) i = (i + 1) & mask;
+        slot[i] = g;
+        return -1;
+    }
+};
+
+// SymmetryAction of the local map `lid` on substate s, from the map tables.
+static inline uint32_t local_image(const HostTables& t, uint32_t lid, uint32_t s) {
+    if (t.m <= 8) return t.lmap_tab[((size_t)lid << t.m) + s];
+    const int hi_n = 1 << (t.m - t.chunk_lo), lo_n = 1 << t.chunk_lo;
+    const uint16_t* tab = &t.lmap_tab[(size_t)lid * (hi_n + lo_n)];
+    return (uint32_t)tab[s >> t.chunk_lo] | (uint32_t)tab[hi_n + (s & (uint32_t)(lo_n - 1))];
 }
 
 ed_status build_host_tables(const ed_sector* sec, HostTables& t) {
@@ -142,20 +182,18 @@ ed_status build_host_tables(const ed_sector* sec, HostTables& t) {
         t.chi_cls[g] = (uint16_t)c;
     }
     // closure and homomorphism
-    std::unordered_map<std::string, int> index;
-    index.reserve((size_t)G * 2);
+    ElemIndex index(t);
     for (int g = 0; g < G; ++g) {
-        auto r = index.emplace(elem_key(&t.perm[(size_t)g * N], N, t.flip[g]), g);
-        if (!r.second) return fail(ED_ERR_NOT_GROUP, "elements %d and %d coincide", r.first->second, g);
+        const int e = index.add(g);
+        if (e >= 0) return fail(ED_ERR_NOT_GROUP, "elements %d and %d coincide", e, g);
     }
     std::vector<int32_t> comp(N);
     for (int a = 0; a < G; ++a) {
         for (int b = 0; b < G; ++b) {
             // (a o b): spin at i moves to perm_b[i], then to perm_a[perm_b[i]]
             for (int i = 0; i < N; ++i) comp[i] = t.perm[(size_t)a * N + t.perm[(size_t)b * N + i]];
-            auto it = index.find(elem_key(comp.data(), N, t.flip[a] ^ t.flip[b]));
-            if (it == index.end()) return fail(ED_ERR_NOT_GROUP, "product of elements %d and %d is missing", a, b);
-            int c = it->second;
+            const int c = index.find(comp.data(), t.flip[a] ^ t.flip[b]);
+            if (c < 0) return fail(ED_ERR_NOT_GROUP, "product of elements %d and %d is missing", a, b);
             double pr = t.chi[2 * a] * t.chi[2 * b] - t.chi[2 * a + 1] * t.chi[2 * b + 1];
             double pi = t.chi[2 * a] * t.chi[2 * b + 1] + t.chi[2 * a + 1] * t.chi[2 * b];
             if (fabs(pr - t.chi[2 * c]) > 1e-9 || fabs(pi - t.chi[2 * c + 1]) > 1e-9)
@@ -179,49 +217,10 @@ ed_status build_host_tables(const ed_sector* sec, HostTables& t) {
         for (int Z = 0; Z < n_sub; ++Z)
             if (!hit[Z]) return fail(ED_ERR_NOT_SUBLATTICE_STABLE, "element %d merges sublattices", g);
     }
-    // SymmetryAction_X(g, s): image of substate s of block X, read in block dest(g, X)
     const int S = 1 << m;
-    t.sa.assign((size_t)G * n_sub * S, 0);
-    for (int g = 0; g < G; ++g)
-        for (int X = 0; X < n_sub; ++X) {
-            const int Z = t.dest[(size_t)g * n_sub + X];
-            uint16_t* row = &t.sa[((size_t)g * n_sub + X) * S];
-            for (int s = 0; s < S; ++s) {
-                uint32_t img = 0;
-                for (int l = 0; l < m; ++l) {
-                    int bit = (s >> (m - 1 - l)) & 1;
-                    if (t.flip[g]) bit ^= 1;
-                    if (bit) {
-                        int lp = t.perm[(size_t)g * N + X * m + l] - Z * m;
-                        img |= 1u << (m - 1 - lp);
-                    }
-                }
-                row[s] = (uint16_t)img;
-            }
-        }
-    // Rep_X and Sym_X over G_X = {g : g maps X onto block 0}
-    t.rep.assign((size_t)n_sub * S, 0xFFFF);
-    t.sym_off.assign((size_t)n_sub * (S + 1), 0);
-    t.sym_ids.clear();
-    for (int X = 0; X < n_sub; ++X) {
-        for (int s = 0; s < S; ++s) {
-            uint32_t best = 0xFFFFFFFFu;
-            for (int g = 0; g < G; ++g)
-                if (t.dest[(size_t)g * n_sub + X] == 0) best = std::min<uint32_t>(best, t.sa[((size_t)g * n_sub + X) * S + s]);
-            t.sym_off[(size_t)X * (S + 1) + s] = (uint32_t)t.sym_ids.size();
-            if (best != 0xFFFFFFFFu) {
-                t.rep[(size_t)X * S + s] = (uint16_t)best;
-                for (int g = 0; g < G; ++g)
-                    if (t.dest[(size_t)g * n_sub + X] == 0 && t.sa[((size_t)g * n_sub + X) * S + s] == best)
-                        t.sym_ids.push_back((uint16_t)g);
-            }
-        }
-        t.sym_off[(size_t)X * (S + 1) + S] = (uint32_t)t.sym_ids.size();
-    }
     // distinct local block maps (positions + flip) and their SymmetryAction tables
     t.chunk_lo = m <= 8 ? 0 : m / 2;
     const int c_lo = t.chunk_lo, c_hi = m - c_lo;
-    const int stride = m <= 8 ? S : (1 << c_hi) + (1 << c_lo);
     std::map<std::vector<int>, int> lmap_id;
     t.srclid.assign((size_t)G * n_sub, 0);
     t.lmap_tab.clear();
@@ -261,7 +260,44 @@ ed_status build_host_tables(const ed_sector* sec, HostTables& t) {
             t.srclid[(size_t)g * n_sub + Z] = (uint32_t)X | ((uint32_t)id << 8);
         }
     t.n_lmap = (int)lmap_id.size();
-    (void)stride;
+    // Rep_X and Sym_X over G_X = {g : g maps X onto block 0}, by the distinct local
+    // maps of G_X (a group of 256 elements has 64 on 16-site blocks): the smallest
+    // image of every substate, the elements whose map reaches it, in order
+    t.rep.assign((size_t)n_sub * S, 0xFFFF);
+    t.sym_off.assign((size_t)n_sub * (S + 1), 0);
+    t.sym_ids.clear();
+    std::vector<uint32_t> pos(S);
+    for (int X = 0; X < n_sub; ++X) {
+        std::vector<std::pair<uint32_t, int>> gx;  // (local map, element)
+        for (int g = 0; g < G; ++g)
+            if (t.dest[(size_t)g * n_sub + X] == 0) gx.push_back({t.srclid[(size_t)g * n_sub] >> 8, g});
+        std::vector<int> n_el(t.n_lmap, 0);
+        for (auto& e : gx) ++n_el[e.first];
+        uint16_t* rep = &t.rep[(size_t)X * S];
+        uint32_t* off = &t.sym_off[(size_t)X * (S + 1)];
+        for (int l = 0; l < t.n_lmap; ++l)
+            if (n_el[l])
+                for (int s = 0; s < S; ++s) rep[s] = std::min(rep[s], (uint16_t)local_image(t, (uint32_t)l, (uint32_t)s));
+        std::vector<std::vector<uint16_t>> reach(t.n_lmap);  // substates a map takes to their smallest image
+        std::fill(pos.begin(), pos.end(), 0u);
+        for (int l = 0; l < t.n_lmap; ++l)
+            if (n_el[l])
+                for (int s = 0; s < S; ++s)
+                    if (local_image(t, (uint32_t)l, (uint32_t)s) == rep[s]) {
+                        reach[l].push_back((uint16_t)s);
+                        pos[s] += (uint32_t)n_el[l];
+                    }
+        uint32_t run = (uint32_t)t.sym_ids.size();
+        for (int s = 0; s < S; ++s) {
+            off[s] = run;
+            run += pos[s];
+            pos[s] = off[s];
+        }
+        off[S] = run;
+        t.sym_ids.resize(run);
+        for (auto& e : gx)
+            for (uint16_t s : reach[e.first]) t.sym_ids[pos[s]++] = (uint16_t)e.second;
+    }
     t.dl.clear();
     t.dl_stride = 0;
     if (t.n_lmap < 4096 && n_sub <= 16) {
@@ -641,7 +677,14 @@ ed_status ed_sector_tables(const ed_sector* sector, uint16_t* rep, uint32_t* sym
     if (sym_off) memcpy(sym_off, t.sym_off.data(), t.sym_off.size() * 4);
     if (sym_ids) memcpy(sym_ids, t.sym_ids.data(), t.sym_ids.size() * 2);
     if (n_sym_ids) *n_sym_ids = (int64_t)t.sym_ids.size();
-    if (sa) memcpy(sa, t.sa.data(), t.sa.size() * 2);
+    if (sa)  // SymmetryAction_X(g, s): image of substate s of block X, read in block dest(g, X)
+        for (int g = 0; g < t.G; ++g)
+            for (int X = 0; X < t.n_sub; ++X) {
+                const int Z = t.dest[(size_t)g * t.n_sub + X], S = 1 << t.m;
+                const uint32_t lid = t.srclid[(size_t)g * t.n_sub + Z] >> 8;
+                uint16_t* row = sa + ((size_t)g * t.n_sub + X) * S;
+                for (int v = 0; v < S; ++v) row[v] = (uint16_t)local_image(t, lid, (uint32_t)v);
+            }
     if (dest) memcpy(dest, t.dest.data(), t.dest.size());
     return ED_OK;
 }

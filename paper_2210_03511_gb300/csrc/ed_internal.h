@@ -57,8 +57,6 @@ struct StreamPool {
 // Table layouts (m = bits per sublattice block, S = 2^m substates):
 //   rep[X*S + s]                 Rep_X(s)                      (Eq. sublatrepdef)
 //   sym_off[X*(S+1) + s .. +1]   range of Sym_X(s) in sym_ids  (Eq. repsymdef)
-//   sa[(g*n_sub + X)*S + s]      SymmetryAction_X(g, s) as an m-bit substate of
-//                                block dest[g*n_sub + X]       (Eq. symactiondef)
 //   src[g*n_sub + Z]             the block X with dest(g, X) = Z
 struct HostTables {
     int N = 0, n_up = 0, G = 0, n_sub = 0, m = 0;
@@ -69,7 +67,6 @@ struct HostTables {
     std::vector<uint16_t> rep;      // [n_sub][S]
     std::vector<uint32_t> sym_off;  // [n_sub][S+1]
     std::vector<uint16_t> sym_ids;
-    std::vector<uint16_t> sa;       // [G][n_sub][S]
     std::vector<uint16_t> chi_cls;  // [G] id of the value chi(g); equal ids <=> equal characters
     bool real_chars = true;
     // SymmetryAction stored once per distinct local block map (a permutation of
