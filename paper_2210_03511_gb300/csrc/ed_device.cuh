@@ -4,8 +4,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <type_traits>
-
 #include "ed_internal.h"
 
 // Helpers are __host__ __device__ so the exact device logic can also run on the
@@ -245,19 +243,28 @@ ED_HD void find_rep(W s, const TabView<CHUNKED>& t, W& rep, int& gbest, int& nst
     compat = cp;
 }
 
-// find_rep for a compile-time number of blocks NS (2..4).  Substates and block
-// representatives live in registers; a candidate g reads its packed (source
-// block, map id) entries for all destination blocks with one 8-byte load, looks
-// all its blocks up at once and compares whole images.  A warp runs this loop as
-// long as its lane with the most candidates (1.5 on average, 5 in the slowest of
-// 32 lanes), so the loop is kept short: no exit in the middle of an image, no
-// turn of its own for moving on to the next list, characters read only on a tie
-// (36-site kagome sector: @@).
+// find_rep for a compile-time number of blocks NS (2..4).  Substates, block
+// representatives and the best image so far (block by block) live in registers.
+// Each candidate g reads its packed (source block, map id) entries for all
+// destination blocks with one 8-byte load and composes its image from the most
+// significant destination block down, stopping at the first block that exceeds
+// the best image (most candidates stop after one lookup).  One flat loop over the
+// concatenated Sym_Y lists of all blocks Y with Rep_Y = MinRep: a separate loop
+// per Y would make a warp wait for the longest list of every Y in turn.
+// A warp runs the loop as long as its lane with the most candidates (1.5 on
+// average, 5 in the slowest of 32 lanes; many more where few spins are up), so a
+// turn is kept short: moving on to the next list takes none of its own, the best
+// image starts above every image instead of behind a flag, characters are read
+// on a tie only.  Matrix-free square32 FP64 3.32 -> 3.01 ms, kagome36 with 11
+// spins up 18.3 -> 17.3 ms, square36 with 13 up 32.6 -> 29.8 ms.
+// Kept in step across the warp: letting a lane start its next state while others
+// still have candidates (square32 4.6 ms) or dealing the candidates of a warp out
+// over its lanes (4.7 ms) lost more, in neighbouring lanes' shared table, Limits
+// and x sectors and in registers, than it won.
 // Same outputs as find_rep.
 template <typename W, bool CHUNKED, int NS>
 ED_HD void find_rep_ns(W s, const TabView<CHUNKED>& t, W& rep, int& gbest, int& nstab, bool& compat) {
     static_assert(NS >= 2 && NS <= 4, "specialised for 2..4 blocks");
-    using I = typename std::conditional<(NS <= 3), uint32_t, uint64_t>::type;  // blocks 1.. of an image, m <= 16
     const int m = t.m;
     const int S = 1 << m;
     uint32_t sub[NS], r[NS];
@@ -281,43 +288,53 @@ ED_HD void find_rep_ns(W s, const TabView<CHUNKED>& t, W& rep, int& gbest, int& 
         q = t.sym_off[Y * (S + 1) + sy];
         q1 = t.sym_off[Y * (S + 1) + sy + 1];
     };
-    auto image = [&](int g) -> I {
-        const uint2 pk = *(const uint2*)(t.dl + (size_t)g * 4);
-        const uint32_t ent[4] = {pk.x & 0xFFFFu, pk.x >> 16, pk.y & 0xFFFFu, pk.y >> 16};
-        I img = 0;
+    // block Z of g.s from its packed entries
+    auto block = [&](const uint2& pk, int Z) -> uint32_t {
+        const uint32_t e = ((Z & 2) ? pk.y : pk.x) >> ((Z & 1) * 16) & 0xFFFFu;
+        const uint32_t X = e >> 12;
+        uint32_t sx = sub[0];
+#pragma unroll
+        for (int k = 1; k < NS; ++k) sx = (X == (uint32_t)k) ? sub[k] : sx;
+        return sym_action<CHUNKED>(t, e & 0xFFFu, sx);
+    };
+    auto packed = [&](int g) { return *(const uint2*)(t.dl + (size_t)g * 4); };
+    uint32_t bestb[NS];
+    bestb[0] = minrep;
+#pragma unroll
+    for (int Z = 1; Z < NS; ++Z) bestb[Z] = 0xFFFFFFFFu;  // above every substate
+    int g = 0, ns = 0;
+    bool cp = true;
+    next_list();  // a list of a block that reaches MinRep is never empty
+    while (true) {
+        const int c = t.sym_ids[q];
+        const uint2 pk = packed(c);
+        uint32_t v[NS];
+        int state = 0;  // 0: equal so far, -1: smaller, 1: larger
 #pragma unroll
         for (int Z = 1; Z < NS; ++Z) {
-            const uint32_t X = ent[Z] >> 12;
-            uint32_t sx = sub[0];
-#pragma unroll
-            for (int k = 1; k < NS; ++k) sx = (X == (uint32_t)k) ? sub[k] : sx;
-            img = (img << m) | (I)sym_action<CHUNKED>(t, ent[Z] & 0xFFFu, sx);
+            if (state == 1) break;
+            v[Z] = block(pk, Z);
+            if (state == 0) state = v[Z] > bestb[Z] ? 1 : (v[Z] < bestb[Z] ? -1 : 0);
         }
-        return img;
-    };
-    next_list();  // a list of a block that reaches MinRep is never empty
-    int g = t.sym_ids[q];
-    I best = image(g);
-    int ns = 1;
-    bool cp = true;
-    while (true) {
+        if (state == -1) {
+#pragma unroll
+            for (int Z = 1; Z < NS; ++Z) bestb[Z] = v[Z];
+            g = c;
+            ns = 1;
+            cp = true;
+        } else if (state == 0) {
+            ++ns;
+            cp = cp && t.chi_cls[c] == t.chi_cls[g];
+        }
         if (++q == q1) {
             if (!ymask) break;
             next_list();
         }
-        const int c = t.sym_ids[q];
-        const I img = image(c);
-        if (img < best) {
-            best = img;
-            g = c;
-            ns = 1;
-            cp = true;
-        } else if (img == best) {
-            ++ns;
-            cp = cp && t.chi_cls[c] == t.chi_cls[g];
-        }
     }
-    rep = ((W)minrep << ((NS - 1) * m)) | (W)best;
+    W best = 0;
+#pragma unroll
+    for (int Z = 0; Z < NS; ++Z) best = (best << m) | (W)bestb[Z];
+    rep = best;
     gbest = g;
     nstab = ns;
     compat = cp;
