@@ -20,6 +20,7 @@
 #include <condition_variable>
 #include <mutex>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "ed_internal.h"
@@ -81,63 +82,176 @@ __device__ __forceinline__ double2 block_sum2(double2 v) {
     return v;  // valid in thread 0
 }
 
-// partial[blockIdx.y * gridDim.x + blockIdx.x] = sum_i conj(A_k[i]) b[i] over this block's slice
-template <int K>
-__global__ void multi_dot(const typename LV<K>::T* A, int64_t ld, const typename LV<K>::T* b, int64_t n,
-                          double2* partial) {
-    const typename LV<K>::T* a = A + (int64_t)blockIdx.y * ld;
-    const int64_t per = (n + gridDim.x - 1) / gridDim.x;
-    const int64_t i0 = (int64_t)blockIdx.x * per, i1 = min(n, i0 + per);
-    double2 acc = make_double2(0, 0);
-    if constexpr (!LV<K>::cplx) {
-        // real vectors: one FP64 FMA per element (FP64 throughput is scarce on this GPU)
-        for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) acc.x += (double)a[i] * (double)b[i];
-    } else {
-        for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-            const double2 x = ld2(a[i]), y = ld2(b[i]);
-            acc.x += x.x * y.x + x.y * y.y;
-            acc.y += x.x * y.y - x.y * y.x;
+// Sums of V values (V = 1, 2, 4 or 8) over the block, the pairs of block_sum2's
+// tree, so the same bits: the first levels halve the number of values a lane
+// carries instead of adding each across the warp (V - 1 + 5 - log2 V additions
+// instead of 5 V).  The result of value q is in thread 8 q of the first two warps.
+template <int V>
+__device__ __forceinline__ double block_sums(double (&v)[V]) {
+    __shared__ double red[V][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int o = 16, q = 0;
+#pragma unroll
+    for (int c = V; c > 1; c /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < c / 2; ++i) {
+            const double keep = up ? v[i + c / 2] : v[i], give = up ? v[i] : v[i + c / 2];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
         }
+        q = 2 * q + (up ? 1 : 0);
     }
-    acc = block_sum2(acc);
-    if (threadIdx.x == 0) partial[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = acc;
+    const int rest = o;
+    for (; o > 0; o /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    __syncthreads();
+    if ((lane & (2 * rest - 1)) == 0) red[q][warp] = v[0];
+    __syncthreads();
+    double r = 0.0;
+    if (threadIdx.x < 8 * V || threadIdx.x < 32) {
+        r = threadIdx.x < 8 * V ? red[threadIdx.x >> 3][threadIdx.x & 7] : 0.0;
+        for (int k = 4; k > 0; k /= 2) r += __shfl_xor_sync(0xffffffffu, r, k);
+    }
+    return r;
 }
 
-// Reorthogonalisation coefficients for FP32 vectors: each thread forms
+// partial[k * gridDim.x + blockIdx.x] = sum_i conj(A_k[i]) b[i] over this block's
+// slice, for J of the vectors (k0 .. k0 + J - 1).  b is read once for them; a
+// complex product keeps its four parts apart (four FP64 operations per element;
+// x.x y.x + x.y y.y added to one sum takes six).
+template <int K, int J>
+__device__ __forceinline__ void dots(const typename LV<K>::T* __restrict__ A, int64_t ld,
+                                     const typename LV<K>::T* __restrict__ b, int64_t i0, int64_t i1, int k0,
+                                     double2* partial) {
+    constexpr int JP = J == 3 ? 4 : J;
+    constexpr int V = LV<K>::cplx ? 2 * JP : JP;
+    double v[V];
+    if constexpr (!LV<K>::cplx) {
+        // real vectors: one FP64 FMA per element (FP64 throughput is scarce on this GPU)
+#pragma unroll
+        for (int j = 0; j < V; ++j) v[j] = 0.0;
+        for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+            const double y = (double)b[i];
+#pragma unroll
+            for (int j = 0; j < J; ++j) v[j] += (double)A[(int64_t)j * ld + i] * y;
+        }
+    } else {
+        double p[J][4];
+#pragma unroll
+        for (int j = 0; j < J; ++j) p[j][0] = p[j][1] = p[j][2] = p[j][3] = 0.0;
+        for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+            const double2 y = ld2(b[i]);
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const double2 x = ld2(A[(int64_t)j * ld + i]);
+                p[j][0] += x.x * y.x;
+                p[j][1] += x.y * y.y;
+                p[j][2] += x.x * y.y;
+                p[j][3] += x.y * y.x;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < JP; ++j) {
+            v[2 * j] = j < J ? p[j < J ? j : 0][0] + p[j < J ? j : 0][1] : 0.0;
+            v[2 * j + 1] = j < J ? p[j < J ? j : 0][2] - p[j < J ? j : 0][3] : 0.0;
+        }
+    }
+    const double r = block_sums<V>(v);
+    constexpr int per = LV<K>::cplx ? 2 : 1;
+    const int q = threadIdx.x >> 3;
+    if ((threadIdx.x & 7) == 0 && q < per * J) {
+        double* out = (double*)(partial + (int64_t)(k0 + q / per) * gridDim.x + blockIdx.x);
+        out[q % per] = r;
+        if (per == 1) out[1] = 0.0;
+    }
+}
+
+// The same for FP32 vectors' reorthogonalisation coefficients: each thread forms
 // partial sums of 16 consecutive products in FP32 and adds them to its FP64
 // accumulator (GB300 has little FP64 throughput).  The coefficients then
 // carry a relative error ~16 eps_32 of sum |x_i y_i|, far below what
 // keeping the Lanczos vectors orthogonal to working precision needs; the
 // Lanczos coefficients alpha and beta keep full FP64 accumulation.
-template <int K>
-__global__ void multi_dot_f32(const typename LV<K>::T* A, int64_t ld, const typename LV<K>::T* b, int64_t n,
-                              double2* partial) {
+template <int K, int J>
+__device__ __forceinline__ void dots_f32(const typename LV<K>::T* __restrict__ A, int64_t ld,
+                                         const typename LV<K>::T* __restrict__ b, int64_t i0, int64_t i1, int k0,
+                                         double2* partial) {
     static_assert(K == 1 || K == 3, "FP32 vectors only");
-    const typename LV<K>::T* a = A + (int64_t)blockIdx.y * ld;
-    const int64_t per = (n + gridDim.x - 1) / gridDim.x;
-    const int64_t i0 = (int64_t)blockIdx.x * per, i1 = min(n, i0 + per);
-    double2 acc = make_double2(0, 0);
-    float cx = 0.f, cy = 0.f;
+    constexpr int JP = J == 3 ? 4 : J;
+    constexpr int per = LV<K>::cplx ? 2 : 1;
+    constexpr int V = per * JP;
+    double v[V];
+    float c[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        v[j] = 0.0;
+        c[j] = 0.f;
+    }
     int cnt = 0;
     for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-        if constexpr (K == 1) {
-            cx = fmaf(a[i], b[i], cx);
-        } else {
-            const float2 x = a[i], y = b[i];
-            cx = fmaf(x.x, y.x, fmaf(x.y, y.y, cx));
-            cy = fmaf(x.x, y.y, fmaf(-x.y, y.x, cy));
+        const auto y = b[i];
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const auto x = A[(int64_t)j * ld + i];
+            if constexpr (K == 1) {
+                c[j] = fmaf(x, y, c[j]);
+            } else {
+                c[2 * j] = fmaf(x.x, y.x, fmaf(x.y, y.y, c[2 * j]));
+                c[2 * j + 1] = fmaf(x.x, y.y, fmaf(-x.y, y.x, c[2 * j + 1]));
+            }
         }
         if (++cnt == 16) {
-            acc.x += (double)cx;
-            acc.y += (double)cy;
-            cx = cy = 0.f;
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                v[j] += (double)c[j];
+                c[j] = 0.f;
+            }
             cnt = 0;
         }
     }
-    acc.x += (double)cx;
-    acc.y += (double)cy;
-    acc = block_sum2(acc);
-    if (threadIdx.x == 0) partial[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = acc;
+#pragma unroll
+    for (int j = 0; j < V; ++j) v[j] += (double)c[j];
+    const double r = block_sums<V>(v);
+    const int q = threadIdx.x >> 3;
+    if ((threadIdx.x & 7) == 0 && q < per * J) {
+        double* out = (double*)(partial + (int64_t)(k0 + q / per) * gridDim.x + blockIdx.x);
+        out[q % per] = r;
+        if (per == 1) out[1] = 0.0;
+    }
+}
+
+// Dots of b with the nk vectors A_k, four to a block row.  Bound by the FP64
+// pipe: one vector to a block row spent 10 of 26 FP64 instructions per warp on
+// the block sums (square32 FP64, 52 steps of full reorthogonalisation: 10.1 ->
+// 8.1 ms; a time-evolution step of 30 complex FP64 vectors there, with
+// multi_axpy: 58.1 -> 46.7 ms).
+template <int K, bool F32>
+__global__ void __launch_bounds__(256) multi_dot_kernel(const typename LV<K>::T* A, int64_t ld, int nk,
+                                                        const typename LV<K>::T* b, int64_t n, double2* partial) {
+    const int k0 = 4 * blockIdx.y, left = nk - k0;
+    const int64_t per = (n + gridDim.x - 1) / gridDim.x;
+    const int64_t i0 = (int64_t)blockIdx.x * per, i1 = min(n, i0 + per);
+    const typename LV<K>::T* a = A + (int64_t)k0 * ld;
+    auto go = [&](auto j) {
+        constexpr int J = decltype(j)::value;
+        if constexpr (F32) dots_f32<K, J>(a, ld, b, i0, i1, k0, partial);
+        else dots<K, J>(a, ld, b, i0, i1, k0, partial);
+    };
+    if (left >= 4) go(std::integral_constant<int, 4>{});
+    else if (left == 3) go(std::integral_constant<int, 3>{});
+    else if (left == 2) go(std::integral_constant<int, 2>{});
+    else go(std::integral_constant<int, 1>{});
+}
+
+template <int K>
+static void multi_dot(const typename LV<K>::T* A, int64_t ld, int nk, const typename LV<K>::T* b, int64_t n,
+                      double2* partial, int nb, cudaStream_t s) {
+    multi_dot_kernel<K, false><<<dim3(nb, (nk + 3) / 4), 256, 0, s>>>(A, ld, nk, b, n, partial);
+}
+
+template <int K>
+static void multi_dot_f32(const typename LV<K>::T* A, int64_t ld, int nk, const typename LV<K>::T* b, int64_t n,
+                          double2* partial, int nb, cudaStream_t s) {
+    multi_dot_kernel<K, true><<<dim3(nb, (nk + 3) / 4), 256, 0, s>>>(A, ld, nk, b, n, partial);
 }
 
 // w -= sum_k c_k A_k in FP32 arithmetic for FP32 vectors (the coefficients
@@ -208,26 +322,50 @@ __global__ void lanczos_axpy(typename LV<K>::T* w, const typename LV<K>::T* v, c
     }
 }
 
-// w -= sum_k c_k A_k  (classical Gram-Schmidt update)
+// w -= sum_k c_k A_k  (classical Gram-Schmidt update), two elements a thread so
+// that the loads of eight vectors' elements are in flight.  Complex products are
+// summed in four parts (four FP64 operations per element instead of six) and
+// subtracted once.
 template <int K>
-__global__ void multi_axpy(typename LV<K>::T* w, const typename LV<K>::T* A, int64_t ld, int nk, const double2* c,
-                           int64_t n) {
-    if constexpr (!LV<K>::cplx) {
-        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-            double x = (double)w[i];
-            for (int k = 0; k < nk; ++k) x -= c[k].x * (double)A[(int64_t)k * ld + i];
-            w[i] = (typename LV<K>::T)x;
-        }
-    } else {
-        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-            double2 x = ld2(w[i]);
+__global__ void __launch_bounds__(256) multi_axpy(typename LV<K>::T* w, const typename LV<K>::T* A, int64_t ld, int nk,
+                                                  const double2* __restrict__ c, int64_t n) {
+    using T = typename LV<K>::T;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += 2 * step) {
+        const bool two = i + step < n;
+        const int64_t j = two ? i + step : i;
+        if constexpr (!LV<K>::cplx) {
+            double x = (double)w[i], y = (double)w[j];
+#pragma unroll 4
             for (int k = 0; k < nk; ++k) {
-                const double2 a = ld2(A[(int64_t)k * ld + i]);
-                const double2 ck = c[k];
-                x.x -= ck.x * a.x - ck.y * a.y;
-                x.y -= ck.x * a.y + ck.y * a.x;
+                const double ck = c[k].x;
+                x -= ck * (double)A[(int64_t)k * ld + i];
+                y -= ck * (double)A[(int64_t)k * ld + j];
             }
+            w[i] = (T)x;
+            if (two) w[j] = (T)y;
+        } else {
+            double p[2][4] = {};
+#pragma unroll 2
+            for (int k = 0; k < nk; ++k) {
+                const double2 ck = c[k];
+                const double2 a0 = ld2(A[(int64_t)k * ld + i]), a1 = ld2(A[(int64_t)k * ld + j]);
+                p[0][0] += ck.x * a0.x;
+                p[0][1] += ck.y * a0.y;
+                p[0][2] += ck.x * a0.y;
+                p[0][3] += ck.y * a0.x;
+                p[1][0] += ck.x * a1.x;
+                p[1][1] += ck.y * a1.y;
+                p[1][2] += ck.x * a1.y;
+                p[1][3] += ck.y * a1.x;
+            }
+            double2 x = ld2(w[i]), y = ld2(w[j]);
+            x.x -= p[0][0] - p[0][1];
+            x.y -= p[0][2] + p[0][3];
+            y.x -= p[1][0] - p[1][1];
+            y.y -= p[1][2] + p[1][3];
             st2(w[i], x);
+            if (two) st2(w[j], y);
         }
     }
 }
@@ -771,7 +909,7 @@ static ed_status run(const ed_hamiltonian* h, const ed_lanczos_opts* o, double* 
     const unsigned g = z.grid();
     auto vec = [&](int k) -> T* { return V + (int64_t)(all_slots ? k : (k % 3)) * D; };
     auto dot = [&](const T* A, int nk, const T* bv, double2* out) {
-        multi_dot<K><<<dim3(z.nb, nk), 256, 0, s>>>(A, D, bv, D, partial);
+        multi_dot<K>(A, D, nk, bv, D, partial, z.nb, s);
         reduce_partials<<<std::min(nk, 1024), 256, 0, s>>>(partial, z.nb, nk, out);
     };
     // v_1: keyed random (or the caller's start vector), normalised
@@ -867,7 +1005,7 @@ static ed_status run(const ed_hamiltonian* h, const ed_lanczos_opts* o, double* 
                 const int nj = n + 1 - j0;
                 const T* Vj = V + (int64_t)j0 * D;
                 if constexpr (K == 1 || K == 3) {
-                    multi_dot_f32<K><<<dim3(z.nb, nj), 256, 0, s>>>(Vj, D, w, D, partial);
+                    multi_dot_f32<K>(Vj, D, nj, w, D, partial, z.nb, s);
                     reduce_partials<<<std::min(nj, 1024), 256, 0, s>>>(partial, z.nb, nj, coef);
                     multi_axpy_f32<K><<<g, 256, 0, s>>>(w, Vj, D, nj, coef, D);
                 } else {
@@ -875,7 +1013,7 @@ static ed_status run(const ed_hamiltonian* h, const ed_lanczos_opts* o, double* 
                     multi_axpy<K><<<g, 256, 0, s>>>(w, Vj, D, nj, coef, D);
                 }
             }
-            multi_dot<K><<<dim3(z.nb, 1), 256, 0, s>>>(w, D, w, D, partial);
+            multi_dot<K>(w, D, 1, w, D, partial, z.nb, s);
             norm_from_partials<<<1, 256, 0, s>>>(partial, z.nb, be_dev + n);
         }
         // v_{n+1} = w / beta_{n+1} (unused when the recursion stops at n); in
@@ -1092,7 +1230,7 @@ static ed_status run(const ed_hamiltonian* h, const ed_lanczos_opts* o, double* 
                 double2* res64 = (double2*)z.get((size_t)3 * nk * sizeof(double2));
                 if (!w64 || !part64 || !res64) return fail(ED_ERR_NOMEM, "refinement workspace");
                 auto dot64 = [&](const T64* a, const T64* b2, double2* out) {
-                    multi_dot<K64><<<dim3(z.nb, 1), 256, 0, s>>>(a, D, b2, D, part64);
+                    multi_dot<K64>(a, D, 1, b2, D, part64, z.nb, s);
                     reduce_partials<<<1, 256, 0, s>>>(part64, z.nb, 1, out);
                 };
                 ed_status st = apply_launch(h, d64, y64, w64, nk, s);
@@ -1193,9 +1331,9 @@ static ed_status expectation_kind(const ed_hamiltonian* h, const void* x, int nv
     if (st != ED_OK) return st;
     const T* xv = (const T*)x;
     for (int v = 0; v < nvec; ++v) {
-        multi_dot<K><<<dim3(z.nb, 1), 256, 0, s>>>(xv + (int64_t)v * D, D, y + (int64_t)v * D, D, partial);
+        multi_dot<K>(xv + (int64_t)v * D, D, 1, y + (int64_t)v * D, D, partial, z.nb, s);
         reduce_partials<<<1, 256, 0, s>>>(partial, z.nb, 1, res + 2 * v);
-        multi_dot<K><<<dim3(z.nb, 1), 256, 0, s>>>(xv + (int64_t)v * D, D, xv + (int64_t)v * D, D, partial);
+        multi_dot<K>(xv + (int64_t)v * D, D, 1, xv + (int64_t)v * D, D, partial, z.nb, s);
         reduce_partials<<<1, 256, 0, s>>>(partial, z.nb, 1, res + 2 * v + 1);
     }
     ED_CUDA(cudaGetLastError());
@@ -1280,7 +1418,7 @@ static ed_status evolve_kind(const ed_hamiltonian* h, void* psi, double dt, int 
     if (!V || !w || !partial || !coef || !beta_d || !alpha_d) return fail(ED_ERR_NOMEM, "time-evolution workspace");
     const unsigned g = z.grid();
     auto dot = [&](const T* A, int nk, const T* bv, double2* out) {
-        multi_dot<K><<<dim3(z.nb, nk), 256, 0, s>>>(A, D, bv, D, partial);
+        multi_dot<K>(A, D, nk, bv, D, partial, z.nb, s);
         reduce_partials<<<std::min(nk, 1024), 256, 0, s>>>(partial, z.nb, nk, out);
     };
     // v_0 = psi / |psi|
@@ -1378,7 +1516,7 @@ static ed_status tridiag_kind(const ed_hamiltonian* h, ed_dtype dt, const void* 
     if (!V || !w || !partial || !coef || !beta_d || !alpha_d) return fail(ED_ERR_NOMEM, "Lanczos workspace");
     const unsigned g = z.grid();
     auto dot = [&](const T* A, int nk, const T* bv, double2* out) {
-        multi_dot<K><<<dim3(z.nb, nk), 256, 0, s>>>(A, D, bv, D, partial);
+        multi_dot<K>(A, D, nk, bv, D, partial, z.nb, s);
         reduce_partials<<<std::min(nk, 1024), 256, 0, s>>>(partial, z.nb, nk, out);
     };
     auto slot = [&](int n) { return V + (int64_t)(reorth ? n : (n & 1)) * D; };
