@@ -341,6 +341,33 @@ static bool maps_close(const std::map<std::vector<int>, double>& A, const std::m
     return true;
 }
 
+// A bond set as a table over site pairs.  A permutation of the sites maps distinct
+// bonds to distinct pairs, so it maps the set onto itself when every bond's image
+// is a bond of the same coupling (to 1e-12 (1 + |J|), as maps_close).
+struct BondTable {
+    int N;
+    std::vector<std::pair<int, int>> list;
+    std::vector<double> J;        // [N][N], both orders
+    std::vector<char> there;
+    BondTable(const std::map<std::vector<int>, double>& bonds, int n)
+        : N(n), J((size_t)n * n, 0.0), there((size_t)n * n, 0) {
+        for (auto& kv : bonds) {
+            const int a = kv.first[0], b = kv.first[1];
+            list.push_back({a, b});
+            J[(size_t)a * N + b] = J[(size_t)b * N + a] = kv.second;
+            there[(size_t)a * N + b] = there[(size_t)b * N + a] = 1;
+        }
+    }
+    bool invariant(const int32_t* p) const {
+        for (auto& e : list) {
+            const size_t at = (size_t)p[e.first] * N + p[e.second];
+            const double from = J[(size_t)e.first * N + e.second], to = J[at];
+            if (!there[at] || fabs(to - from) > 1e-12 * (1.0 + fabs(to))) return false;
+        }
+        return true;
+    }
+};
+
 static ed_status prepare_terms(const ed_basis* b, const ed_terms* tm, ed_hamiltonian* h) {
     const HostTables& t = b->ht;
     const int N = t.N;
@@ -365,21 +392,20 @@ static ed_status prepare_terms(const ed_basis* b, const ed_terms* tm, ed_hamilto
     }
     // invariance under every element (spin flip is a pi rotation in spin space:
     // it leaves both S.S and the scalar triple product unchanged)
+    const BondTable bt(bonds, N);
     for (int g = 0; g < t.G; ++g) {
         const int32_t* p = &t.perm[(size_t)g * N];
-        std::map<std::vector<int>, double> b2, t2;
-        for (auto& kv : bonds) {
-            int a, c;
-            canon_bond(p[kv.first[0]], p[kv.first[1]], a, c);
-            b2[{a, c}] += kv.second;
+        bool same = bt.invariant(p);
+        if (same && !tris.empty()) {
+            std::map<std::vector<int>, double> t2;
+            for (auto& kv : tris) {
+                int key[3], sg;
+                canon_tri(p[kv.first[0]], p[kv.first[1]], p[kv.first[2]], key, sg);
+                t2[{key[0], key[1], key[2]}] += sg * kv.second;
+            }
+            same = maps_close(tris, t2);
         }
-        for (auto& kv : tris) {
-            int key[3], sg;
-            canon_tri(p[kv.first[0]], p[kv.first[1]], p[kv.first[2]], key, sg);
-            t2[{key[0], key[1], key[2]}] += sg * kv.second;
-        }
-        if (!maps_close(bonds, b2) || !maps_close(tris, t2))
-            return fail(ED_ERR_NOT_SYMMETRIC, "element %d does not map the terms onto themselves", g);
+        if (!same) return fail(ED_ERR_NOT_SYMMETRIC, "element %d does not map the terms onto themselves", g);
     }
     // Ising part grouped by coupling
     std::map<double, std::vector<std::pair<int, int>>> cls;
@@ -477,15 +503,9 @@ static ed_status prepare_terms_sun(const ed_basis* b, const ed_terms* tm, ed_ham
         canon_bond(i, j, a, c);
         bonds[{a, c}] += tm->J[q];
     }
+    const BondTable bt(bonds, N);
     for (int g = 0; g < G; ++g) {
-        const int32_t* p = &b->sun_perm[(size_t)g * N];
-        std::map<std::vector<int>, double> b2;
-        for (auto& kv : bonds) {
-            int a, c;
-            canon_bond(p[kv.first[0]], p[kv.first[1]], a, c);
-            b2[{a, c}] += kv.second;
-        }
-        if (!maps_close(bonds, b2)) return fail(ED_ERR_NOT_SYMMETRIC, "element %d does not map the terms onto themselves", g);
+        if (!bt.invariant(&b->sun_perm[(size_t)g * N])) return fail(ED_ERR_NOT_SYMMETRIC, "element %d does not map the terms onto themselves", g);
     }
     h->flips.clear();
     std::vector<double> vals;
@@ -520,24 +540,31 @@ static ed_status prepare_terms_sun(const ed_basis* b, const ed_terms* tm, ed_ham
 }
 
 static ed_status upload_terms(const ed_basis* basis, ed_hamiltonian* h) {
-    const Alloc& A = basis->alloc;
-    auto up = [&](DevBuf& d, const void* src, size_t bytes) -> bool {
-        d.bytes = bytes ? bytes : 16;
-        d.p = A.get(d.bytes, 0);
-        if (!d.p) return false;
-        if (bytes && cudaMemcpy(d.p, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) return false;
-        return true;
+    // one allocation and one copy
+    struct Part {
+        DevBuf* d;
+        const void* src;
+        size_t bytes;
     };
-    bool ok = up(h->d_flips, h->flips.data(), h->flips.size() * sizeof(FlipTerm)) &&
-              up(h->d_diag_pos, h->diag_pos.data(), h->diag_pos.size()) &&
-              up(h->d_diag_cls, h->diag_cls.data(), h->diag_cls.size() * sizeof(DiagClass)) &&
-              up(h->d_jhs, h->jhs.data(), h->jhs.size() * sizeof(double)) &&
-              up(h->d_jcls, h->jcls.data(), h->jcls.size());
-    if (ok) {
-        h->d_counters.bytes = 32;
-        h->d_counters.p = A.get(32, 0);
-        ok = h->d_counters.p && cudaMemset(h->d_counters.p, 0, 32) == cudaSuccess;
+    const Part parts[] = {{&h->d_flips, h->flips.data(), h->flips.size() * sizeof(FlipTerm)},
+                          {&h->d_diag_pos, h->diag_pos.data(), h->diag_pos.size()},
+                          {&h->d_diag_cls, h->diag_cls.data(), h->diag_cls.size() * sizeof(DiagClass)},
+                          {&h->d_jhs, h->jhs.data(), h->jhs.size() * sizeof(double)},
+                          {&h->d_jcls, h->jcls.data(), h->jcls.size()},
+                          {&h->d_counters, nullptr, 32}};
+    std::vector<uint8_t> image;
+    std::vector<size_t> at;
+    for (const Part& p : parts) {
+        at.push_back(image.size());
+        image.resize((image.size() + std::max<size_t>(p.bytes, 16) + 255) & ~(size_t)255, 0);
+        if (p.src && p.bytes) memcpy(&image[at.back()], p.src, p.bytes);
     }
+    h->d_terms.bytes = image.size();
+    h->d_terms.p = basis->alloc.get(image.size(), 0);
+    const bool ok =
+        h->d_terms.p && cudaMemcpy(h->d_terms.p, image.data(), image.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+    if (ok)
+        for (size_t i = 0; i < at.size(); ++i) parts[i].d->p = (uint8_t*)h->d_terms.p + at[i];
     return ok ? ED_OK : fail(ED_ERR_NOMEM, "device allocation for terms failed");
 }
 
@@ -780,12 +807,7 @@ void ed_hamiltonian_free(ed_hamiltonian* h) {
     if (!h) return;
     cache_free(h);
     const Alloc& A = h->basis->alloc;
-    A.put(h->d_flips.p, h->d_flips.bytes, 0);
-    A.put(h->d_diag_pos.p, h->d_diag_pos.bytes, 0);
-    A.put(h->d_diag_cls.p, h->d_diag_cls.bytes, 0);
-    A.put(h->d_counters.p, h->d_counters.bytes, 0);
-    A.put(h->d_jhs.p, h->d_jhs.bytes, 0);
-    A.put(h->d_jcls.p, h->d_jcls.bytes, 0);
+    A.put(h->d_terms.p, h->d_terms.bytes, 0);
     delete h;
 }
 

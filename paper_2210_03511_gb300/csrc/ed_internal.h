@@ -182,6 +182,7 @@ struct ed_hamiltonian {
     std::vector<ed::FlipTerm> flips;
     std::vector<int8_t> diag_pos;       // [2*n_diag_bonds] bit positions
     std::vector<ed::DiagClass> diag_cls;
+    ed::DevBuf d_terms;                 // one allocation: the arrays below are parts of it
     ed::DevBuf d_flips, d_diag_pos, d_diag_cls, d_counters;
     int n_diag_cls = 0;
     // real coefficients: jhs[c][n] = jhalf_c * sqrt(n) for the distinct jhalf values c
