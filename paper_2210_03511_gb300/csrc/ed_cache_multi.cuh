@@ -3,13 +3,14 @@
 //
 // With the vectors one after another each element gathers a 32-byte sector per
 // vector.  So x is first copied to [row][NP] (NP = 2, 4 or 8 >= NV vectors): all
-// vectors' x_j of an element lie in one run.  Bound by the L1 data pipe (two
-// loads of up to 32 bytes per lane).  square32, copy included, against one
-// one-vector pass after another: two real vectors 0.30 against 0.49 ms, five
-// 0.71 against 1.22, eight 0.81 against 1.95 (at first, one kernel gathering
-// vector by vector: five in 1.81 ms).  FP64 vectors take one-vector passes: they
-// are bound by the FP64 pipe, and the copy won nothing (square32, three vectors:
-// 0.94 against 1.00 ms real, 1.85 against 1.82 complex).
+// vectors' x_j of an element lie in one run.  Bound by the L1 data pipe.
+// square32, copy included, against one one-vector pass after another: two real
+// vectors 0.31 against 0.49 ms, five 0.58 against 1.22, eight 0.58 against 1.95,
+// five complex 1.34 (one lane per row: five 0.71, eight 0.81, five complex 1.62;
+// at first, one kernel gathering vector by vector: five in 1.81 ms).  FP64 vectors
+// take one-vector passes: they are bound by the FP64 pipe, and the copy won
+// nothing (square32, three vectors: 0.94 against 1.00 ms real, 1.85 against 1.82
+// complex).
 // The sums are those of the one-vector pass, entry by entry.
 #pragma once
 
@@ -22,33 +23,76 @@ namespace ed {
 template <int NV>
 constexpr int padded = NV <= 2 ? 2 : (NV <= 4 ? 4 : 8);
 
-// The first NV of a row's NP elements, in loads of 16 bytes and a shorter last one.
+// A row of more than 16 bytes is read in two halves by two neighbouring lanes, each
+// taking its half of the rows of both lanes one after another: the lanes of a load
+// then share sectors, where one lane reading its whole row fetches every sector
+// twice and more through the L1 data pipe.  (Four lanes to a 64-byte row were
+// slower: five complex vectors 2.09 against 1.34 ms.)
 template <typename T, int NV>
-struct Row {
-    T v[NV];
+struct Layout {
+    static constexpr int NP = padded<NV>;
+    static constexpr int G = NP * sizeof(T) <= 16 ? 1 : 2;
+    static constexpr int P = NP / G;  // elements of a lane's part
 };
 
 template <typename T, int NV>
-__device__ __forceinline__ Row<T, NV> load_row(const T* __restrict__ p) {
-    constexpr int bytes = NV * (int)sizeof(T);
-    constexpr int full = bytes / 16, rest = bytes % 16;
+struct Parts {
+    T v[Layout<T, NV>::G][Layout<T, NV>::P];  // [row of the group][element of this lane's part]
+    uint32_t w[Layout<T, NV>::G];             // the rows' entry words
+};
+
+template <typename T, int P>
+__device__ __forceinline__ void load_part(T (&v)[P], const T* __restrict__ p) {
+    constexpr int n = P * (int)sizeof(T) / 16;
     union {
-        uint4 q[(bytes + 15) / 16];
-        Row<T, NV> r;
+        uint4 q[n ? n : 1];
+        uint2 d;
+        T e[P];
     } u;
+    if constexpr (n == 0) u.d = __ldg((const uint2*)p);
 #pragma unroll
-    for (int i = 0; i < full; ++i) u.q[i] = __ldg((const uint4*)p + i);
-    if constexpr (rest == 4) {
-        u.q[full].x = __ldg((const unsigned*)((const uint4*)p + full));
-    } else if constexpr (rest == 8) {
-        const uint2 e = __ldg((const uint2*)((const uint4*)p + full));
-        u.q[full].x = e.x;
-        u.q[full].y = e.y;
-    } else if constexpr (rest == 12) {
-        u.q[full] = __ldg((const uint4*)p + full);  // the fourth is the padding of NP = 4 or 8
-    }
-    return u.r;
+    for (int i = 0; i < n; ++i) u.q[i] = __ldg((const uint4*)p + i);
+#pragma unroll
+    for (int j = 0; j < P; ++j) v[j] = u.e[j];
 }
+
+// The sums of one slice: this lane's part of the rows of its group.
+template <int K, int NV>
+struct GroupSum {
+    using T = typename Val<K>::T;
+    using R = typename Val<K>::R;
+    using L = Layout<T, NV>;
+    RowSum<K, false> sum[L::G][L::P];
+
+    template <typename Coef>
+    __device__ __forceinline__ void run(uint32_t c, const uint32_t* ent, const T* __restrict__ xs, uint32_t ob, int lane,
+                                        Coef&& coef) {
+        constexpr int bytes = L::NP * (int)sizeof(T);
+        constexpr int ahead = bytes > 16 ? 2 : AHEAD;
+        const uint32_t om = (1u << ob) - 1u;
+        const int h = lane % L::G, l0 = lane - h;
+        walk<Parts<T, NV>, ahead, true>(
+            c, ent, 0u, 255u, lane,
+            [&](uint32_t w) {
+                Parts<T, NV> x;
+#pragma unroll
+                for (int r = 0; r < L::G; ++r) {
+                    x.w[r] = L::G == 1 ? w : __shfl_sync(FULL, w, l0 + r);
+                    load_part<T, L::P>(x.v[r], xs + (int64_t)(x.w[r] & om) * L::NP + h * L::P);
+                }
+                return x;
+            },
+            [&](uint32_t, const Parts<T, NV>& x, unsigned has) {
+#pragma unroll
+                for (int r = 0; r < L::G; ++r) {
+                    if (!((has >> (l0 + r)) & 1u)) continue;
+                    const auto cf = coef(x.w[r] >> ob);
+#pragma unroll
+                    for (int j = 0; j < L::P; ++j) sum[r][j].add(cf, false, x.v[r][j]);
+                }
+            });
+    }
+};
 
 // xi[i][NP] = row i of the vectors of all sectors (one sector: row_off null).
 template <typename T, int NP>
@@ -81,11 +125,8 @@ __global__ void interleave_kernel(T* __restrict__ xi, const T* __restrict__ x, i
     }
 }
 
-// entries in flight: about 64 bytes of gathered x per lane, at most AHEAD
 template <typename T, int NV>
-constexpr int multi_ahead = NV * sizeof(T) > 32 ? 1 : (NV * sizeof(T) > 16 ? 2 : AHEAD);
-template <typename T, int NV>
-constexpr int multi_blocks = NV * sizeof(T) > 32 ? 2 : (NV * sizeof(T) > 16 ? 3 : 4);
+constexpr int multi_blocks = Layout<T, NV>::NP * sizeof(T) > 32 ? 2 : 4;  // five real vectors 0.58 ms against 0.64 (3)
 
 template <int K, int NV>
 __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>) cache_pass_multi(CachePass p) {
@@ -93,16 +134,17 @@ __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>) c
     using T = typename V::T;
     using R = typename V::R;
     using CT = typename std::conditional<V::cplx, T, R>::type;
-    constexpr int NP = padded<NV>;
+    using L = Layout<T, NV>;
+    constexpr int NP = L::NP;
     __shared__ CT ctab[NCODE];
     stage_codes<K>(ctab, p.ctab);
     write_counters(p);
     __syncthreads();
     const T* __restrict__ xi = (const T*)p.xi;
     T* __restrict__ y = (T*)p.y;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, h = lane % L::G;
     const int64_t D = p.D;
-    const uint32_t ob = p.off_bits, om = (1u << ob) - 1u;
+    const uint32_t ob = p.off_bits;
     const bool last = p.mode == 0 || p.mode == 3, prev = p.mode >= 2;
     const T* __restrict__ xs = xi + p.xoff * NP;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -113,31 +155,36 @@ __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>) c
         const uint32_t c = nx.c;
         const uint32_t* ent = nx.base + nx.bo;
         if (sl + warps < p.ns) nx.load(p, sl + warps, lane);
-        const int64_t row = sl * NSLICE + lane;
-        const bool keep = row < D && (c > 0 || last || !prev);  // the row's y is written
-        RowSum<K, false> sum[NV];
+        const int64_t first = sl * NSLICE + lane - h;  // the group's rows
+        bool keep[L::G];                               // whose y is written
+        GroupSum<K, NV> group;
 #pragma unroll
-        for (int v = 0; v < NV; ++v)
-            if (prev && keep) sum[v].start(y[(int64_t)v * D + row]);
-        walk<Row<T, NV>, multi_ahead<T, NV>>(
-            c, ent, 0u, 255u, lane, [&](uint32_t w) { return load_row<T, NV>(xs + (int64_t)(w & om) * NP); },
-            [&](uint32_t w, const Row<T, NV>& xj) {
-                const CT cf = ctab[w >> ob];
+        for (int r = 0; r < L::G; ++r) {
+            const uint32_t cr = L::G == 1 ? c : __shfl_sync(FULL, c, lane - h + r);
+            keep[r] = first + r < D && (cr > 0 || last || !prev);
 #pragma unroll
-                for (int v = 0; v < NV; ++v) sum[v].add(cf, false, xj.v[v]);
-            });
-        if (!keep) continue;
-        R inv = 0, dg = 0;
-        Row<T, NV> xr;
-        if (last) {
-            inv = ((const R*)p.isq)[__ldg(p.stab + row)];
-            dg = (R)__ldg(p.diag + row);
-            xr = load_row<T, NV>(xi + row * NP);
+            for (int j = 0; j < L::P; ++j)
+                if (prev && keep[r] && h * L::P + j < NV) group.sum[r][j].start(y[(int64_t)(h * L::P + j) * D + first + r]);
         }
+        group.run(c, ent, xs, ob, lane, [&](uint32_t cd) { return ctab[cd]; });
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            sum[v].close();
-            finish<K>(y + (int64_t)v * D + row, &xr.v[v], sum[v].re, sum[v].im, last, inv, dg);
+        for (int r = 0; r < L::G; ++r) {
+            if (!keep[r]) continue;
+            const int64_t row = first + r;
+            R inv = 0, dg = 0;
+            T xr[L::P];
+            if (last) {
+                inv = ((const R*)p.isq)[__ldg(p.stab + row)];
+                dg = (R)__ldg(p.diag + row);
+                load_part<T, L::P>(xr, xi + row * NP + h * L::P);
+            }
+#pragma unroll
+            for (int j = 0; j < L::P; ++j) {
+                if (h * L::P + j >= NV) continue;
+                RowSum<K, false>& sm = group.sum[r][j];
+                sm.close();
+                finish<K>(y + (int64_t)(h * L::P + j) * D + row, &xr[j], sm.re, sm.im, last, inv, dg);
+            }
         }
     }
 }
@@ -152,8 +199,9 @@ __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>)
     using T = typename V::T;
     using R = typename V::R;
     using CT = typename std::conditional<V::cplx, T, R>::type;
-    constexpr int NP = padded<NV>;
-    const int lane = threadIdx.x & 31;
+    using L = Layout<T, NV>;
+    constexpr int NP = L::NP;
+    const int lane = threadIdx.x & 31, h = lane % L::G;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t gs = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); gs < n_slices; gs += warps) {
         int lo = 0, hi = n_sec - 1;
@@ -171,24 +219,24 @@ __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>)
         const R* __restrict__ isq;
         if constexpr (K == 0 || K == 2) isq = (const R*)c.sq + c.G1;
         else isq = (const R*)c.sqf + c.G1;
-        const uint32_t ob = c.off_bits, om = (1u << ob) - 1u;
-        RowSum<K, false> sum[NV];
-        walk<Row<T, NV>, multi_ahead<T, NV>>(
-            __ldg(c.counts + row), c.ent[ls >> c.chunk_shift] + __ldg(c.boff + ls), 0u, 255u, lane,
-            [&](uint32_t w) { return load_row<T, NV>(xi + (int64_t)(w & om) * NP); },
-            [&](uint32_t w, const Row<T, NV>& xj) {
-                const CT cf = __ldg(ctab + (V::cplx ? 1 : 2) * (w >> ob));
+        GroupSum<K, NV> group;
+        group.run(__ldg(c.counts + row), c.ent[ls >> c.chunk_shift] + __ldg(c.boff + ls), xi, c.off_bits, lane,
+               [&](uint32_t cd) { return __ldg(ctab + (V::cplx ? 1 : 2) * cd); });
 #pragma unroll
-                for (int v = 0; v < NV; ++v) sum[v].add(cf, false, xj.v[v]);
-            });
-        if (row >= D) continue;
-        const R inv = isq[__ldg(c.stab + row)];
-        const R dg = (R)__ldg(c.diag + row);
-        const Row<T, NV> xr = load_row<T, NV>(xi + row * NP);
+        for (int r = 0; r < L::G; ++r) {
+            const int64_t at = row - h + r;
+            if (at >= D) continue;
+            const R inv = isq[__ldg(c.stab + at)];
+            const R dg = (R)__ldg(c.diag + at);
+            T xr[L::P];
+            load_part<T, L::P>(xr, xi + at * NP + h * L::P);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            sum[v].close();
-            finish<K>(y + (int64_t)v * D + row, &xr.v[v], sum[v].re, sum[v].im, true, inv, dg);
+            for (int j = 0; j < L::P; ++j) {
+                if (h * L::P + j >= NV) continue;
+                RowSum<K, false>& sm = group.sum[r][j];
+                sm.close();
+                finish<K>(y + (int64_t)(h * L::P + j) * D + at, &xr[j], sm.re, sm.im, true, inv, dg);
+            }
         }
     }
 }

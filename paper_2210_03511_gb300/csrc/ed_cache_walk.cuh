@@ -12,8 +12,10 @@ constexpr int AHEAD = 4;   // entries in flight per lane (measured: ed_cache_pas
 // Walk entries [k0, k1) of every row of a slice in order (c: entries of this
 // lane's row; p: the slice's first entry; k0, k1 and p uniform over the warp).
 // get(w) loads x for entry word w, use(w, x) adds it.  Once a row of the slice
-// has ended, the places of the others' entries come from ballots.
-template <typename X, int U, typename Get, typename Use>
+// has ended, the places of the others' entries come from ballots.  ALL: both are
+// called by the whole warp, use with the mask of the lanes that have an entry
+// (the others' word is 0).
+template <typename X, int U, bool ALL = false, typename Get, typename Use>
 __device__ __forceinline__ void walk(uint32_t c, const uint32_t* p, uint32_t k0, uint32_t k1, int lane, Get&& get,
                                      Use&& use) {
     const uint32_t cmin = __reduce_min_sync(FULL, c);
@@ -30,27 +32,33 @@ __device__ __forceinline__ void walk(uint32_t c, const uint32_t* p, uint32_t k0,
 #pragma unroll
         for (int u = 0; u < U; ++u) xv[u] = get(w[u]);
 #pragma unroll
-        for (int u = 0; u < U; ++u) use(w[u], xv[u]);
+        for (int u = 0; u < U; ++u) {
+            if constexpr (ALL) use(w[u], xv[u], FULL);
+            else use(w[u], xv[u]);
+        }
     }
     const unsigned lt = (1u << lane) - 1u;
     for (; k < k1; k += U) {
         uint32_t w[U];
         X xv[U];
         bool has[U];
+        unsigned m[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             has[u] = c > k + u && k + u < k1;
-            const unsigned m = __ballot_sync(FULL, has[u]);
+            m[u] = __ballot_sync(FULL, has[u]);
             w[u] = 0;
-            if (has[u]) w[u] = __ldg(q + __popc(m & lt));
-            q += __popc(m);
+            if (has[u]) w[u] = __ldg(q + __popc(m[u] & lt));
+            q += __popc(m[u]);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (has[u]) xv[u] = get(w[u]);
+            if (ALL || has[u]) xv[u] = get(w[u]);
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (has[u]) use(w[u], xv[u]);
+        for (int u = 0; u < U; ++u) {
+            if constexpr (ALL) use(w[u], xv[u], m[u]);
+            else if (has[u]) use(w[u], xv[u]);
+        }
     }
 }
 
