@@ -101,8 +101,8 @@ ed_status apply_batch_launch(const BatchLaunch& L, cudaStream_t s) {
 }
 
 ed_status apply_launch(const ed_hamiltonian* h, ed_dtype dt, const void* x, void* y, int nvec, cudaStream_t s,
-                       bool use_cache) {
-    if (use_cache && h->cache.valid) return cache_apply(h, dt, x, y, nvec, s);
+                       bool use_cache, bool diff) {
+    if (use_cache && h->cache.valid) return cache_apply(h, dt, x, y, nvec, s, diff);
     if (h->sun)
         return fail(ED_ERR_ARG, "an SU(N) Hamiltonian is applied through its stored structure, which was released");
     const ed_basis* b = h->basis;

@@ -679,7 +679,8 @@ ed_status cache_build(ed_hamiltonian* h, ed_dtype dtype, int seg_log2, size_t ma
     return st;
 }
 
-ed_status cache_apply(const ed_hamiltonian* h, ed_dtype dt, const void* x, void* y, int nvec, cudaStream_t s) {
+ed_status cache_apply(const ed_hamiltonian* h, ed_dtype dt, const void* x, void* y, int nvec, cudaStream_t s,
+                      bool diff) {
     const HCache& c = h->cache;
     const ed_basis* b = h->basis;
     CachePass p{};
@@ -692,6 +693,7 @@ ed_status cache_apply(const ed_hamiltonian* h, ed_dtype dt, const void* x, void*
     p.D = b->dim;
     p.ns = c.ns;
     p.nvec = nvec;
+    p.diff = diff;
     p.n_ent = c.n_ent;
     p.n_skip = c.n_skip;
     p.off_bits = (uint32_t)c.off_bits;

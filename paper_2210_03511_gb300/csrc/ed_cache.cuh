@@ -27,6 +27,7 @@ struct CachePass {
     const uint16_t* stab;       // [D] |Stab sigma_i|
     const double* diag;         // [D] Ising part
     int64_t D, ns, xoff;        // xoff: first column of the segment
+    bool diff;                  // general complex sums by product differences (RowSum)
     int nvec, mode;             // mode 0: the only segment, 1: first, 2: inner, 3: last
     int chunk_shift;            // slice >> chunk_shift = chunk
     uint32_t off_bits;          // entry = (code << off_bits) | column offset

@@ -42,7 +42,7 @@ constexpr int pass_blocks(int K) { return K == 2 ? 3 : 5; }
 // compile-time flag so that the one-segment pass carries no such register.  A
 // row's sum continues from that partial sum; a row without entries in an inner
 // segment is left alone.
-template <int K, bool AX, bool PREV>
+template <int K, bool AX, bool PREV, bool DIFF>
 __global__ void __launch_bounds__(BLOCK, pass_blocks(K)) cache_pass_kernel(CachePass p) {
     using V = Val<K>;
     using T = typename V::T;
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(BLOCK, pass_blocks(K)) cache_pass_kernel(Cache
         if (sl + warps < p.ns) nx.load(p, sl + warps, lane);
         const int64_t row = sl * NSLICE + lane;
         const bool keep = row < D && (c > 0 || last || !PREV);  // the row's y is written
-        RowSum<K, AX> sum;
+        RowSum<K, AX, DIFF> sum;
         if (PREV && keep) sum.start(y[row]);
         walk<T, AHEAD>(
             c, ent, 0u, 255u, lane, [&](uint32_t w) { return xs[w & om]; },
@@ -205,12 +205,12 @@ __global__ void __launch_bounds__(BLOCK, pass_blocks(K))
     }
 }
 
-template <int K, bool AX>
+template <int K, bool AX, bool DIFF = false>
 ed_status launch_pass(const CachePass& p, int sms, cudaStream_t s) {
     const int64_t need = (p.ns + (BLOCK / 32) - 1) / (BLOCK / 32);
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sms * pass_blocks(K)));
-    if (p.mode >= 2) cache_pass_kernel<K, AX, true><<<grid, BLOCK, 0, s>>>(p);
-    else cache_pass_kernel<K, AX, false><<<grid, BLOCK, 0, s>>>(p);
+    if (p.mode >= 2) cache_pass_kernel<K, AX, true, DIFF><<<grid, BLOCK, 0, s>>>(p);
+    else cache_pass_kernel<K, AX, false, DIFF><<<grid, BLOCK, 0, s>>>(p);
     ED_CUDA(cudaGetLastError());
     return ED_OK;
 }
@@ -247,7 +247,9 @@ ed_status launch_kind(const CachePass& p, bool ax, int lanes, int sms, cudaStrea
             }
             continue;
         }
-        if constexpr (Val<K>::cplx) st = ax ? launch_pass<K, true>(q, sms, s) : launch_pass<K, false>(q, sms, s);
+        if constexpr (Val<K>::cplx)
+            st = ax ? launch_pass<K, true>(q, sms, s)
+                    : (p.diff ? launch_pass<K, false, true>(q, sms, s) : launch_pass<K, false>(q, sms, s));
         else st = launch_pass<K, false>(q, sms, s);
     }
     return st;

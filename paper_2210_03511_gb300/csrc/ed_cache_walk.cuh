@@ -62,6 +62,10 @@ __device__ __forceinline__ void walk(uint32_t c, const uint32_t* p, uint32_t k0,
     }
 }
 
+// a b rounded, never fused with what follows
+__device__ __forceinline__ double prod(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float prod(float a, float b) { return __fmul_rn(a, b); }
+
 // Sum of one row for one vector of kind K.  AX (complex kinds): every code's
 // coefficient is real or purely imaginary (real characters: Heisenberg terms
 // real, chirality terms imaginary), so one entry costs two real multiply-adds
@@ -75,11 +79,14 @@ __device__ __forceinline__ void walk(uint32_t c, const uint32_t* p, uint32_t k0,
 // its own size, so the rounding errors stay those of the difference added in one
 // go (4.2 against 4.5 10^-16, 5.6 against 5.7 of |y| on kagome sectors); two
 // multiply-adds into one sum round it twice.
-template <int K, bool AX>
+// DIFF: the fused difference of products, added in one go, all the same (for
+// ed_lanczos: the sign of a Ritz vector hangs on the last bits of alpha and beta,
+// so its recursion keeps the arithmetic that its vectors have had).
+template <int K, bool AX, bool DIFF = false>
 struct RowSum {
     using T = typename Val<K>::T;
     using R = typename Val<K>::R;
-    static constexpr bool four = Val<K>::cplx && !AX;
+    static constexpr bool four = Val<K>::cplx && !AX && !DIFF;
     R re = 0, im = 0, re2 = 0, im2 = 0;
     __device__ __forceinline__ void start(const T& y) {
         if constexpr (Val<K>::cplx) {
@@ -96,6 +103,9 @@ struct RowSum {
         } else if constexpr (AX) {
             re += cf.x * (imag ? x.y : x.x);
             im += cf.y * (imag ? x.x : x.y);
+        } else if constexpr (DIFF) {
+            re += fma(cf.x, x.x, -prod(cf.y, x.y));
+            im += fma(cf.y, x.x, prod(cf.x, x.y));
         } else {
             re += cf.x * x.x;
             re2 += cf.y * x.y;

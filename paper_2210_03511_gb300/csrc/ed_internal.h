@@ -284,10 +284,11 @@ ed_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, uint
                              cudaStream_t s);
 // implemented in ed_apply.cu; uses the stored structure when there is one and use_cache is set
 ed_status apply_launch(const ed_hamiltonian* h, ed_dtype dt, const void* x, void* y, int nvec, cudaStream_t s,
-                       bool use_cache = true);
+                       bool use_cache = true, bool diff = false);  // diff: RowSum (ed_cache_walk.cuh)
 // implemented in ed_cache.cu
 ed_status cache_build(ed_hamiltonian* h, ed_dtype dtype, int seg_log2, size_t max_bytes, cudaStream_t s);
-ed_status cache_apply(const ed_hamiltonian* h, ed_dtype dt, const void* x, void* y, int nvec, cudaStream_t s);
+ed_status cache_apply(const ed_hamiltonian* h, ed_dtype dt, const void* x, void* y, int nvec, cudaStream_t s,
+                      bool diff = false);
 void cache_free(ed_hamiltonian* h);
 // implemented in ed_lanczos.cu
 void tridiag_lowest(const std::vector<double>& a, const std::vector<double>& b, int n, int k, bool filter,

@@ -136,7 +136,8 @@ __device__ __forceinline__ double block_sums(double (&v)[V]) {
 // slice, for J of the vectors (k0 .. k0 + J - 1).  b is read once for them; a
 // complex product keeps its four parts apart (four FP64 operations per element;
 // x.x y.x + x.y y.y added to one sum takes six).
-template <int K, int J>
+// DIFF: the one sum per part all the same (ed_lanczos, see RowSum).
+template <int K, int J, bool DIFF>
 __device__ __forceinline__ void dots(const typename LV<K>::T* __restrict__ A, int64_t ld,
                                      const typename LV<K>::T* __restrict__ b, int64_t i0, int64_t i1, int k0,
                                      double2* partial) {
@@ -151,6 +152,18 @@ __device__ __forceinline__ void dots(const typename LV<K>::T* __restrict__ A, in
             const double y = widen(b[i]);
 #pragma unroll
             for (int j = 0; j < J; ++j) v[j] += widen(A[(int64_t)j * ld + i]) * y;
+        }
+    } else if constexpr (DIFF) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) v[j] = 0.0;
+        for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+            const double2 y = ld2(b[i]);
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const double2 x = ld2(A[(int64_t)j * ld + i]);
+                v[2 * j] += x.x * y.x + x.y * y.y;
+                v[2 * j + 1] += x.x * y.y - x.y * y.x;
+            }
         }
     } else {
         double p[J][4];
@@ -242,7 +255,7 @@ __device__ __forceinline__ void dots_f32(const typename LV<K>::T* __restrict__ A
 // the block sums (square32 FP64, 52 steps of full reorthogonalisation: 10.1 ->
 // 8.1 ms; a time-evolution step of 30 complex FP64 vectors there, with
 // multi_axpy: 58.1 -> 46.7 ms).
-template <int K, bool F32>
+template <int K, bool F32, bool DIFF>
 __global__ void __launch_bounds__(256) multi_dot_kernel(const typename LV<K>::T* A, int64_t ld, int nk,
                                                         const typename LV<K>::T* b, int64_t n, double2* partial) {
     const int k0 = 4 * blockIdx.y, left = nk - k0;
@@ -252,7 +265,7 @@ __global__ void __launch_bounds__(256) multi_dot_kernel(const typename LV<K>::T*
     auto go = [&](auto j) {
         constexpr int J = decltype(j)::value;
         if constexpr (F32) dots_f32<K, J>(a, ld, b, i0, i1, k0, partial);
-        else dots<K, J>(a, ld, b, i0, i1, k0, partial);
+        else dots<K, J, DIFF>(a, ld, b, i0, i1, k0, partial);
     };
     if (left >= 4) go(std::integral_constant<int, 4>{});
     else if (left == 3) go(std::integral_constant<int, 3>{});
@@ -260,16 +273,16 @@ __global__ void __launch_bounds__(256) multi_dot_kernel(const typename LV<K>::T*
     else go(std::integral_constant<int, 1>{});
 }
 
-template <int K>
+template <int K, bool DIFF = false>
 static void multi_dot(const typename LV<K>::T* A, int64_t ld, int nk, const typename LV<K>::T* b, int64_t n,
                       double2* partial, int nb, cudaStream_t s) {
-    multi_dot_kernel<K, false><<<dim3(nb, (nk + 3) / 4), 256, 0, s>>>(A, ld, nk, b, n, partial);
+    multi_dot_kernel<K, false, DIFF><<<dim3(nb, (nk + 3) / 4), 256, 0, s>>>(A, ld, nk, b, n, partial);
 }
 
 template <int K>
 static void multi_dot_f32(const typename LV<K>::T* A, int64_t ld, int nk, const typename LV<K>::T* b, int64_t n,
                           double2* partial, int nb, cudaStream_t s) {
-    multi_dot_kernel<K, true><<<dim3(nb, (nk + 3) / 4), 256, 0, s>>>(A, ld, nk, b, n, partial);
+    multi_dot_kernel<K, true, false><<<dim3(nb, (nk + 3) / 4), 256, 0, s>>>(A, ld, nk, b, n, partial);
 }
 
 // w -= sum_k c_k A_k in FP32 arithmetic for FP32 vectors (the coefficients
@@ -343,8 +356,8 @@ __global__ void lanczos_axpy(typename LV<K>::T* w, const typename LV<K>::T* v, c
 // w -= sum_k c_k A_k  (classical Gram-Schmidt update), two elements a thread so
 // that the loads of eight vectors' elements are in flight.  Complex products are
 // summed in four parts (four FP64 operations per element instead of six) and
-// subtracted once.
-template <int K>
+// subtracted once (DIFF: vector by vector, ed_lanczos, see RowSum).
+template <int K, bool DIFF = false>
 __global__ void __launch_bounds__(256) multi_axpy(typename LV<K>::T* w, const typename LV<K>::T* A, int64_t ld, int nk,
                                                   const double2* __restrict__ c, int64_t n) {
     using T = typename LV<K>::T;
@@ -362,6 +375,19 @@ __global__ void __launch_bounds__(256) multi_axpy(typename LV<K>::T* w, const ty
             }
             w[i] = (T)x;
             if (two) w[j] = (T)y;
+        } else if constexpr (DIFF) {
+            double2 x = ld2(w[i]), y = ld2(w[j]);
+#pragma unroll 2
+            for (int k = 0; k < nk; ++k) {
+                const double2 ck = c[k];
+                const double2 a0 = ld2(A[(int64_t)k * ld + i]), a1 = ld2(A[(int64_t)k * ld + j]);
+                x.x -= ck.x * a0.x - ck.y * a0.y;
+                x.y -= ck.x * a0.y + ck.y * a0.x;
+                y.x -= ck.x * a1.x - ck.y * a1.y;
+                y.y -= ck.x * a1.y + ck.y * a1.x;
+            }
+            st2(w[i], x);
+            if (two) st2(w[j], y);
         } else {
             double p[2][4] = {};
 #pragma unroll 2
@@ -928,7 +954,7 @@ static ed_status run(const ed_hamiltonian* h, const ed_lanczos_opts* o, double* 
     const unsigned g = z.grid();
     auto vec = [&](int k) -> T* { return V + (int64_t)(all_slots ? k : (k % 3)) * D; };
     auto dot = [&](const T* A, int nk, const T* bv, double2* out) {
-        multi_dot<K>(A, D, nk, bv, D, partial, z.nb, s);
+        multi_dot<K, true>(A, D, nk, bv, D, partial, z.nb, s);
         reduce_partials<<<std::min(nk, 1024), 256, 0, s>>>(partial, z.nb, nk, out);
     };
     // v_1: keyed random (or the caller's start vector), normalised
@@ -1004,7 +1030,7 @@ static ed_status run(const ed_hamiltonian* h, const ed_lanczos_opts* o, double* 
     ED_CUDA(cudaEventCreateWithFlags(&ph.ev[1], cudaEventDisableTiming));
     const unsigned gs = (unsigned)std::max<int64_t>(1, std::min<int64_t>((D + 255) / 256, 1024));
     auto enqueue = [&](int n) -> ed_status {
-        ed_status st = apply_launch(h, vdt, vec(n), w, 1, s);
+        ed_status st = apply_launch(h, vdt, vec(n), w, 1, s, true, true);
         if (st != ED_OK) return st;
         ++n_apply;
         const T* vp = n > 0 ? vec(n - 1) : nullptr;
@@ -1029,10 +1055,10 @@ static ed_status run(const ed_hamiltonian* h, const ed_lanczos_opts* o, double* 
                     multi_axpy_f32<K><<<g, 256, 0, s>>>(w, Vj, D, nj, coef, D);
                 } else {
                     dot(Vj, nj, w, coef);
-                    multi_axpy<K><<<g, 256, 0, s>>>(w, Vj, D, nj, coef, D);
+                    multi_axpy<K, true><<<g, 256, 0, s>>>(w, Vj, D, nj, coef, D);
                 }
             }
-            multi_dot<K>(w, D, 1, w, D, partial, z.nb, s);
+            multi_dot<K, true>(w, D, 1, w, D, partial, z.nb, s);
             norm_from_partials<<<1, 256, 0, s>>>(partial, z.nb, be_dev + n);
         }
         // v_{n+1} = w / beta_{n+1} (unused when the recursion stops at n); in
@@ -1180,7 +1206,7 @@ static ed_status run(const ed_hamiltonian* h, const ed_lanczos_opts* o, double* 
             if (nacc) accumulate<K, T><<<g, 256, 0, s>>>((T*)evecs, D, nacc, cj, vec(j), D);
             if (y64) accumulate<K, T64><<<g, 256, 0, s>>>(y64, D, ny, cj + nacc, vec(j), D);
             if (j + 1 == iters) break;
-            ed_status st = apply_launch(h, vdt, vec(j), w, 1, s);
+            ed_status st = apply_launch(h, vdt, vec(j), w, 1, s, true, true);
             if (st != ED_OK) return st;
             ++n_apply;
             lanczos_axpy<K><<<g, 256, 0, s>>>(w, vec(j), j > 0 ? vec(j - 1) : nullptr, D, al_d + j,
@@ -1249,10 +1275,10 @@ static ed_status run(const ed_hamiltonian* h, const ed_lanczos_opts* o, double* 
                 double2* res64 = (double2*)z.get((size_t)3 * nk * sizeof(double2));
                 if (!w64 || !part64 || !res64) return fail(ED_ERR_NOMEM, "refinement workspace");
                 auto dot64 = [&](const T64* a, const T64* b2, double2* out) {
-                    multi_dot<K64>(a, D, 1, b2, D, part64, z.nb, s);
+                    multi_dot<K64, true>(a, D, 1, b2, D, part64, z.nb, s);
                     reduce_partials<<<1, 256, 0, s>>>(part64, z.nb, 1, out);
                 };
-                ed_status st = apply_launch(h, d64, y64, w64, nk, s);
+                ed_status st = apply_launch(h, d64, y64, w64, nk, s, true, true);
                 if (st != ED_OK) return st;
                 n_apply += nk;
                 std::vector<double2> hres(2 * (size_t)nk);
