@@ -256,9 +256,9 @@ __device__ __forceinline__ void dots_f32(const typename LV<K>::T* __restrict__ A
 // 8.1 ms; a time-evolution step of 30 complex FP64 vectors there, with
 // multi_axpy: 58.1 -> 46.7 ms).
 template <int K, bool F32, bool DIFF>
-__global__ void __launch_bounds__(256) multi_dot_kernel(const typename LV<K>::T* A, int64_t ld, int nk,
+__global__ void __launch_bounds__(256) multi_dot_kernel(const typename LV<K>::T* A, int64_t ld, int nk, int rows,
                                                         const typename LV<K>::T* b, int64_t n, double2* partial) {
-    const int k0 = 4 * blockIdx.y, left = nk - k0;
+    const int k0 = rows * blockIdx.y, left = min(rows, nk - k0);
     const int64_t per = (n + gridDim.x - 1) / gridDim.x;
     const int64_t i0 = (int64_t)blockIdx.x * per, i1 = min(n, i0 + per);
     const typename LV<K>::T* a = A + (int64_t)k0 * ld;
@@ -273,16 +273,24 @@ __global__ void __launch_bounds__(256) multi_dot_kernel(const typename LV<K>::T*
     else go(std::integral_constant<int, 1>{});
 }
 
+// Vectors per block row: four where that leaves two blocks for each of 152 SMs, else
+// one (a sector of 28,699 rows has 8 slices; with four to a row always, and two elements
+// a thread in multi_axpy, the 36 triangular24 sectors one by one took 0.94 s, now
+// 0.77, at first 0.80).
+static int dot_rows(int nb, int nk) { return (int64_t)nb * ((nk + 3) / 4) >= 304 ? 4 : 1; }
+
 template <int K, bool DIFF = false>
 static void multi_dot(const typename LV<K>::T* A, int64_t ld, int nk, const typename LV<K>::T* b, int64_t n,
                       double2* partial, int nb, cudaStream_t s) {
-    multi_dot_kernel<K, false, DIFF><<<dim3(nb, (nk + 3) / 4), 256, 0, s>>>(A, ld, nk, b, n, partial);
+    const int rows = dot_rows(nb, nk);
+    multi_dot_kernel<K, false, DIFF><<<dim3(nb, (nk + rows - 1) / rows), 256, 0, s>>>(A, ld, nk, rows, b, n, partial);
 }
 
 template <int K>
 static void multi_dot_f32(const typename LV<K>::T* A, int64_t ld, int nk, const typename LV<K>::T* b, int64_t n,
                           double2* partial, int nb, cudaStream_t s) {
-    multi_dot_kernel<K, true, false><<<dim3(nb, (nk + 3) / 4), 256, 0, s>>>(A, ld, nk, b, n, partial);
+    const int rows = dot_rows(nb, nk);
+    multi_dot_kernel<K, true, false><<<dim3(nb, (nk + rows - 1) / rows), 256, 0, s>>>(A, ld, nk, rows, b, n, partial);
 }
 
 // w -= sum_k c_k A_k in FP32 arithmetic for FP32 vectors (the coefficients
@@ -353,65 +361,77 @@ __global__ void lanczos_axpy(typename LV<K>::T* w, const typename LV<K>::T* v, c
     }
 }
 
-// w -= sum_k c_k A_k  (classical Gram-Schmidt update), two elements a thread so
-// that the loads of eight vectors' elements are in flight.  Complex products are
-// summed in four parts (four FP64 operations per element instead of six) and
-// subtracted once (DIFF: vector by vector, ed_lanczos, see RowSum).
-template <int K, bool DIFF = false>
-__global__ void __launch_bounds__(256) multi_axpy(typename LV<K>::T* w, const typename LV<K>::T* A, int64_t ld, int nk,
-                                                  const double2* __restrict__ c, int64_t n) {
+// w -= sum_k c_k A_k  (classical Gram-Schmidt update), E elements a thread at a
+// time.  Complex products are summed in four parts (four FP64 operations per
+// element instead of six) and subtracted once (DIFF: vector by vector, ed_lanczos,
+// see RowSum).
+template <int K, bool DIFF, int E>
+__global__ void __launch_bounds__(256) multi_axpy_kernel(typename LV<K>::T* w, const typename LV<K>::T* A, int64_t ld,
+                                                         int nk, const double2* __restrict__ c, int64_t n) {
     using T = typename LV<K>::T;
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += 2 * step) {
-        const bool two = i + step < n;
-        const int64_t j = two ? i + step : i;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += E * step) {
+        int64_t at[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) at[e] = i + e * step < n ? i + e * step : i;
         if constexpr (!LV<K>::cplx) {
-            double x = widen(w[i]), y = widen(w[j]);
+            double x[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) x[e] = widen(w[at[e]]);
 #pragma unroll 4
             for (int k = 0; k < nk; ++k) {
                 const double ck = c[k].x;
-                x -= ck * widen(A[(int64_t)k * ld + i]);
-                y -= ck * widen(A[(int64_t)k * ld + j]);
+#pragma unroll
+                for (int e = 0; e < E; ++e) x[e] -= ck * widen(A[(int64_t)k * ld + at[e]]);
             }
-            w[i] = (T)x;
-            if (two) w[j] = (T)y;
-        } else if constexpr (DIFF) {
-            double2 x = ld2(w[i]), y = ld2(w[j]);
-#pragma unroll 2
-            for (int k = 0; k < nk; ++k) {
-                const double2 ck = c[k];
-                const double2 a0 = ld2(A[(int64_t)k * ld + i]), a1 = ld2(A[(int64_t)k * ld + j]);
-                x.x -= ck.x * a0.x - ck.y * a0.y;
-                x.y -= ck.x * a0.y + ck.y * a0.x;
-                y.x -= ck.x * a1.x - ck.y * a1.y;
-                y.y -= ck.x * a1.y + ck.y * a1.x;
-            }
-            st2(w[i], x);
-            if (two) st2(w[j], y);
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (i + e * step < n) w[at[e]] = (T)x[e];
         } else {
-            double p[2][4] = {};
+            double2 x[E];
+            double p[E][4] = {};
+            if constexpr (DIFF) {
+#pragma unroll
+                for (int e = 0; e < E; ++e) x[e] = ld2(w[at[e]]);
+            }
 #pragma unroll 2
             for (int k = 0; k < nk; ++k) {
                 const double2 ck = c[k];
-                const double2 a0 = ld2(A[(int64_t)k * ld + i]), a1 = ld2(A[(int64_t)k * ld + j]);
-                p[0][0] += ck.x * a0.x;
-                p[0][1] += ck.y * a0.y;
-                p[0][2] += ck.x * a0.y;
-                p[0][3] += ck.y * a0.x;
-                p[1][0] += ck.x * a1.x;
-                p[1][1] += ck.y * a1.y;
-                p[1][2] += ck.x * a1.y;
-                p[1][3] += ck.y * a1.x;
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const double2 a = ld2(A[(int64_t)k * ld + at[e]]);
+                    if constexpr (DIFF) {
+                        x[e].x -= ck.x * a.x - ck.y * a.y;
+                        x[e].y -= ck.x * a.y + ck.y * a.x;
+                    } else {
+                        p[e][0] += ck.x * a.x;
+                        p[e][1] += ck.y * a.y;
+                        p[e][2] += ck.x * a.y;
+                        p[e][3] += ck.y * a.x;
+                    }
+                }
             }
-            double2 x = ld2(w[i]), y = ld2(w[j]);
-            x.x -= p[0][0] - p[0][1];
-            x.y -= p[0][2] + p[0][3];
-            y.x -= p[1][0] - p[1][1];
-            y.y -= p[1][2] + p[1][3];
-            st2(w[i], x);
-            if (two) st2(w[j], y);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                if (i + e * step >= n) continue;
+                if constexpr (!DIFF) {
+                    x[e] = ld2(w[at[e]]);
+                    x[e].x -= p[e][0] - p[e][1];
+                    x[e].y -= p[e][2] + p[e][3];
+                }
+                st2(w[at[e]], x[e]);
+            }
         }
     }
+}
+
+// Two elements a thread where the grid does not cover the vector anyway (a second
+// one that repeats the first would double the FP64 work of a small sector).
+template <int K, bool DIFF = false>
+static void multi_axpy(typename LV<K>::T* w, const typename LV<K>::T* A, int64_t ld, int nk, const double2* c, int64_t n,
+                       unsigned g, cudaStream_t s) {
+    if (n > (int64_t)g * 256) multi_axpy_kernel<K, DIFF, 2><<<g, 256, 0, s>>>(w, A, ld, nk, c, n);
+    else multi_axpy_kernel<K, DIFF, 1><<<g, 256, 0, s>>>(w, A, ld, nk, c, n);
 }
 
 // out = sum_k s_k A_k with real coefficients s (FP64 accumulation, output type O)
@@ -1055,7 +1075,7 @@ static ed_status run(const ed_hamiltonian* h, const ed_lanczos_opts* o, double* 
                     multi_axpy_f32<K><<<g, 256, 0, s>>>(w, Vj, D, nj, coef, D);
                 } else {
                     dot(Vj, nj, w, coef);
-                    multi_axpy<K, true><<<g, 256, 0, s>>>(w, Vj, D, nj, coef, D);
+                    multi_axpy<K, true>(w, Vj, D, nj, coef, D, g, s);
                 }
             }
             multi_dot<K, true>(w, D, 1, w, D, partial, z.nb, s);
@@ -1487,7 +1507,7 @@ static ed_status evolve_kind(const ed_hamiltonian* h, void* psi, double dt, int 
             const int j0 = pass == 0 ? 0 : std::max(0, n - 1);
             const int nj = n + 1 - j0;
             dot(V + (int64_t)j0 * D, nj, w, coef);
-            multi_axpy<K><<<g, 256, 0, s>>>(w, V + (int64_t)j0 * D, D, nj, coef, D);
+            multi_axpy<K>(w, V + (int64_t)j0 * D, D, nj, coef, D, g, s);
         }
         dot(w, 1, w, coef + m + 1);
         sqrt_re<<<1, 1, 0, s>>>(coef + m + 1, beta_d);
@@ -1586,7 +1606,7 @@ static ed_status tridiag_kind(const ed_hamiltonian* h, ed_dtype dt, const void* 
                 const int j0 = pass == 0 ? 0 : std::max(0, n - 1);
                 const int nj = n + 1 - j0;
                 dot(V + (int64_t)j0 * D, nj, w, coef);
-                multi_axpy<K><<<g, 256, 0, s>>>(w, V + (int64_t)j0 * D, D, nj, coef, D);
+                multi_axpy<K>(w, V + (int64_t)j0 * D, D, nj, coef, D, g, s);
             }
         }
         dot(w, 1, w, coef + slots + 1);
