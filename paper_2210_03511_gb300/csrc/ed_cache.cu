@@ -32,10 +32,10 @@
 // Build.  Rows are taken in chunks: one search pass writes every entry of the
 // chunk as (column, coefficient key) to scratch and counts entries per row and
 // segment; the slices' offsets are scanned, the chunk's entries allocated and
-// packed.  Searching costs far more than the 24 bytes of
-// scratch traffic per entry (36-site kagome sector: 165 ms a search of 4.7 10^9
-// entries, against 20 ms), so one search and a pack replace the two searches
-// (count, then fill) that a layout without scratch needs.
+// packed.  Searching costs far more than the 16 bytes of scratch traffic per
+// entry, so one search and a pack (36-site kagome sector, 4.7 10^9 entries: 159
+// and 30 ms) replace the two searches (count, then fill) that a layout without
+// scratch needs.
 #include <math.h>
 
 #include <algorithm>
@@ -752,11 +752,11 @@ extern "C" void ed_hamiltonian_store_free(ed_hamiltonian* h) {
     ed::cache_free(h);
 }
 
-// Segment-size autotuner: a segment of x must stay in L2 while its pass
+// Segment-size autotuner: a segment of x should stay in L2 while its pass
 // gathers from it, but every pass also reads each row's count and updates its
-// partial sum, so fewer, larger segments pay where rows are many (the 40-site
-// square sector prefers 128 MB of FP64) and smaller ones where the gathers
-// dominate (the 36-site kagome sector, complex FP32, prefers 64 MB).
+// partial sum, and short rows leave more of a warp idle, so fewer, larger segments
+// pay where rows are many (the 40-site square sector and the 36-site kagome sector,
+// FP64 and FP32, take 2^24 elements).
 extern "C" ed_status ed_hamiltonian_store_set_lanes(ed_hamiltonian* h, int32_t lanes_per_row) {
     using namespace ed;
     if (!h) return fail(ED_ERR_ARG, "null argument");
