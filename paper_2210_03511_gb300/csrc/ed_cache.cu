@@ -696,6 +696,7 @@ ed_status cache_apply(const ed_hamiltonian* h, ed_dtype dt, const void* x, void*
     p.diff = diff;
     p.n_ent = c.n_ent;
     p.n_skip = c.n_skip;
+    p.nb = c.nb;
     p.off_bits = (uint32_t)c.off_bits;
     p.n_re = (uint32_t)c.n_re;
     const int K = dt == ED_F64 ? 0 : dt == ED_F32 ? 1 : dt == ED_C128 ? 2 : 3;

@@ -34,6 +34,7 @@ struct CachePass {
     uint32_t n_re;              // codes below n_re have real coefficients (complex kinds)
     unsigned long long* counters;  // receives n_ent, n_skip, 0 (ed_apply_counters), or null
     unsigned long long n_ent, n_skip;
+    int nb;                     // segments
 };
 
 // One segment's pass for p.nvec vectors of kind K, `lanes` warps per slice for

@@ -38,12 +38,23 @@ namespace {
 // against 1.66 (4 blocks), square32's complex sector 1.19 against 1.21.
 constexpr int pass_blocks(int K) { return K == 2 ? 3 : 5; }
 
+// Real FP32 vectors over several segments: a row has few entries per segment, so a
+// warp spends its time on starting slices, and eight blocks (32 registers, nothing
+// spilled, the same four entries in flight) hide that better than five.  Against
+// five blocks, by entries per row and segment: square40 138.7 -> 126.3 ms (3.2) and
+// 126.9 -> 118.5 (6.3), square36 12.3 -> 12.0 (4.6), 10.4 -> 9.6 (9.3) and
+// 9.26 -> 8.90 (18.5), square32 0.652 -> 0.654 (3.7), 0.449 -> 0.430 (7.3) and
+// 0.309 -> 0.304 (22).  Below three it loses: square36 16.9 -> 17.6 (2.4), square32
+// 1.00 -> 1.06 (1.8).
+constexpr int MANY_BLOCKS = 8;
+constexpr uint64_t MANY_ROW_ENTRIES = 3;
+
 // PREV: modes 2 and 3 (a partial sum from earlier segments exists in y), a
 // compile-time flag so that the one-segment pass carries no such register.  A
 // row's sum continues from that partial sum; a row without entries in an inner
 // segment is left alone.
-template <int K, bool AX, bool PREV, bool DIFF>
-__global__ void __launch_bounds__(BLOCK, pass_blocks(K)) cache_pass_kernel(CachePass p) {
+template <int K, bool AX, bool PREV, bool DIFF, int BLOCKS>
+__global__ void __launch_bounds__(BLOCK, BLOCKS) cache_pass_kernel(CachePass p) {
     using V = Val<K>;
     using T = typename V::T;
     using R = typename V::R;
@@ -205,12 +216,15 @@ __global__ void __launch_bounds__(BLOCK, pass_blocks(K))
     }
 }
 
-template <int K, bool AX, bool DIFF = false>
+template <int K, bool AX, bool DIFF = false, int BLOCKS = pass_blocks(K)>
 ed_status launch_pass(const CachePass& p, int sms, cudaStream_t s) {
+    if constexpr (K == 1 && BLOCKS != MANY_BLOCKS)
+        if (p.mode != 0 && p.n_ent >= MANY_ROW_ENTRIES * (uint64_t)p.D * (uint64_t)p.nb)
+            return launch_pass<K, AX, DIFF, MANY_BLOCKS>(p, sms, s);
     const int64_t need = (p.ns + (BLOCK / 32) - 1) / (BLOCK / 32);
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sms * pass_blocks(K)));
-    if (p.mode >= 2) cache_pass_kernel<K, AX, true, DIFF><<<grid, BLOCK, 0, s>>>(p);
-    else cache_pass_kernel<K, AX, false, DIFF><<<grid, BLOCK, 0, s>>>(p);
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sms * BLOCKS));
+    if (p.mode >= 2) cache_pass_kernel<K, AX, true, DIFF, BLOCKS><<<grid, BLOCK, 0, s>>>(p);
+    else cache_pass_kernel<K, AX, false, DIFF, BLOCKS><<<grid, BLOCK, 0, s>>>(p);
     ED_CUDA(cudaGetLastError());
     return ED_OK;
 }

@@ -78,3 +78,25 @@ def test_slice_edges(P, name, segments):
         h.store(seg_log2=seg, max_bytes=size - 1)
     assert e.value.name == "ED_ERR_NOMEM"
     assert h.store_info() == dict(entries=0, segments=0, codes=0, bytes=0)
+
+
+@pytest.mark.parametrize("segments", [2, 3, 8])
+@pytest.mark.parametrize("name", sorted(set(CASES) - {"complex"}))
+def test_real_fp32_over_segments(P, name, segments):
+    """One real FP32 vector over several segments, with more and with fewer than three
+    entries per row and segment (two kernels): 64 eps (|H| |x|)_i of FP32."""
+    import torch
+    p = CASES[name][1]()
+    b = P.Basis(p.sector)
+    h = P.Hamiltonian(b, p.terms)
+    reps, stab = oracle.basis(p.sector)
+    H = oracle.csr(p, reps, stab)
+    x32 = state_vector(37, reps, complex_=False).astype(np.float32)
+    x = torch.tensor(x32, device="cuda")
+    y = torch.full_like(x, float("nan"))
+    h.store(P.ED_F32, seg_log2=max(5, int(math.ceil(math.log2(max(b.dim, 2) / segments)))))
+    h.apply(x, y)
+    torch.cuda.synchronize()
+    X = x32.astype(np.float64)
+    bound = 64 * np.finfo(np.float32).eps * (abs(H) @ np.abs(X)) + 1e-30
+    assert np.all(np.abs(y.cpu().numpy().astype(np.float64) - H @ X) <= bound)
