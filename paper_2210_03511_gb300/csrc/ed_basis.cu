@@ -728,6 +728,10 @@ void make_blob(const HostTables& t, DevTables& d, std::vector<uint8_t>& h) {
     d.off_chif = al((size_t)t.G * 8);
     d.off_sqrtf = al((size_t)2 * (t.G + 1) * 4);
     d.dl_stride = t.dl_stride;
+    d.to_block0 = 0;
+    for (int g = 0; g < t.G; ++g)
+        for (int X = 0; X < t.n_sub && X < 32; ++X)
+            if (t.dest[(size_t)g * t.n_sub + X] == 0) d.to_block0 |= 1u << X;
     d.off_dl = al(std::max<size_t>(t.dl.size(), 1) * 2);
     d.off_chineg = al((size_t)t.G);
     const size_t total = (off + 15) & ~(size_t)15;

@@ -50,6 +50,7 @@ struct TabView {
     const uint16_t* dl;       // [G][dl_stride] (dest block << 12) | map id, by source block
     const uint8_t* chi_neg;   // [G] real chi(g) < 0
     int n_sub, m, G, c_lo, stride, dl_stride;
+    uint32_t to_block0;       // bit X: some element maps block X onto block 0
 };
 
 template <bool CHUNKED>
@@ -75,6 +76,7 @@ ED_HD TabView<CHUNKED> tab_view(const uint8_t* base, const DevTables& d) {
     v.dl = (const uint16_t*)(base + d.off_dl);
     v.chi_neg = (const uint8_t*)(base + d.off_chineg);
     v.dl_stride = d.dl_stride;
+    v.to_block0 = d.to_block0;
     return v;
 }
 
@@ -278,6 +280,9 @@ ED_HD void find_rep_ns(W s, const TabView<CHUNKED>& t, W& rep, int& gbest, int& 
     uint32_t ymask = 0;  // blocks Y with Rep_Y = MinRep whose Sym_Y list is still to come
 #pragma unroll
     for (int Y = 0; Y < NS; ++Y) ymask |= (r[Y] == minrep ? 1u : 0u) << Y;
+    // A block that no element maps onto block 0 has empty lists, and the Rep marker
+    // 0xFFFF, which a full 16-site block has too; block 0 has the identity in every list.
+    ymask &= t.to_block0;
     uint32_t q = 0, q1 = 0;
     auto next_list = [&]() {
         const int Y = ctz32(ymask);
@@ -304,7 +309,7 @@ ED_HD void find_rep_ns(W s, const TabView<CHUNKED>& t, W& rep, int& gbest, int& 
     for (int Z = 1; Z < NS; ++Z) bestb[Z] = 0xFFFFFFFFu;  // above every substate
     int g = 0, ns = 0;
     bool cp = true;
-    next_list();  // a list of a block that reaches MinRep is never empty
+    next_list();  // never empty: the lists left in ymask hold at least one element
     while (true) {
         const int c = t.sym_ids[q];
         const uint2 pk = packed(c);

@@ -101,6 +101,7 @@ struct DevTables {
     int lmap_stride;                // entries per map
     uint32_t off_dl, off_chineg;
     int dl_stride;
+    uint32_t to_block0;             // bit X: some element maps block X onto block 0 (X < 32)
 };
 
 // ---------------------------------------------------------------- flip terms (host + device)
