@@ -152,7 +152,7 @@ __device__ __forceinline__ void stage_codes(CT* dst, const void* src) {
 }
 
 __device__ __forceinline__ void write_counters(const CachePass& p) {
-    if (p.counters && blockIdx.x == 0 && threadIdx.x == 0) {
+    if (p.counters && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
         p.counters[0] = p.n_ent;
         p.counters[1] = p.n_skip;
         p.counters[2] = 0ull;
