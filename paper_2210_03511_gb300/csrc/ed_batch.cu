@@ -765,6 +765,9 @@ static BatchLaunch make_launch(const ed_batch* B, ed_dtype dt, const void* x, vo
     ed_status st;
     L.stored = stored_descs(B, st);
     L.stored_slices = B->stored_slices;
+    L.stored_entries = 0;
+    if (L.stored)
+        for (const ed_hamiltonian* h : B->hs) L.stored_entries += h->cache.n_ent;
     return L;
 }
 

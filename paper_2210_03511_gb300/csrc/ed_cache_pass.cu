@@ -49,11 +49,29 @@ constexpr int pass_blocks(int K) { return K == 2 ? 3 : 5; }
 constexpr int MANY_BLOCKS = 8;
 constexpr uint64_t MANY_ROW_ENTRIES = 3;
 
+// Launches of one segment with no more blocks than this per SM, and rows of twice as
+// many entries as these on average: no warp waits for its turn, so a row's chain of
+// entry and x_j loads bounds the call, and twice the entries in flight shorten it.
+// Against four in flight, triangular24 (28,699 rows of 75 entries): real FP32 14.4 ->
+// 12.3 us, FP64 16.8 -> 14.4, complex FP32 20.6 -> 16.4, FP64 24.6 -> 18.5; two complex
+// FP32 vectors 20.6 -> 16.5; a batch of 2,506 real rows 10.3 -> 9.1, 12.3 -> 10.3 (FP64).
+// The same sums in the same order.  Shorter rows have nothing to load ahead (chain16,
+// 8.5 entries: 7.2 -> 7.6 us), and with more blocks the registers cost residents that
+// the call needs.  Sixteen in flight at two blocks gained no more in these sectors
+// (FP64 16.7 us).
+constexpr int few_blocks(int K) { return K == 2 ? 2 : 3; }
+constexpr int FEW_AHEAD = 8;
+template <int K>
+bool few(int64_t slices, int nvec, uint64_t entries, int64_t rows, int sms) {
+    const int64_t blocks = (slices + (BLOCK / 32) - 1) / (BLOCK / 32) * nvec;
+    return blocks <= (int64_t)sms * few_blocks(K) && entries >= 2 * FEW_AHEAD * (uint64_t)rows;
+}
+
 // PREV: modes 2 and 3 (a partial sum from earlier segments exists in y), a
 // compile-time flag so that the one-segment pass carries no such register.  A
 // row's sum continues from that partial sum; a row without entries in an inner
 // segment is left alone.  Vector blockIdx.y of p.nvec.
-template <int K, bool AX, bool PREV, bool DIFF, int BLOCKS>
+template <int K, bool AX, bool PREV, bool DIFF, int BLOCKS, int U>
 __global__ void __launch_bounds__(BLOCK, BLOCKS) cache_pass_kernel(CachePass p) {
     using V = Val<K>;
     using T = typename V::T;
@@ -83,7 +101,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCKS) cache_pass_kernel(CachePass p) 
         const bool keep = row < D && (c > 0 || last || !PREV);  // the row's y is written
         RowSum<K, AX, DIFF> sum;
         if (PREV && keep) sum.start(y[row]);
-        walk<T, AHEAD>(
+        walk<T, U>(
             c, ent, 0u, 255u, lane, [&](uint32_t w) { return xs[w & om]; },
             [&](uint32_t w, const T& xj) {
                 const uint32_t cd = w >> ob;
@@ -170,8 +188,8 @@ __global__ void __launch_bounds__(BLOCK, pass_blocks(K)) cache_pass_split(CacheP
 // Vectors are those of a batch: sector s's nvec columns start at element
 // nvec * row_off[s].  x may advance by x_step_elems per device-side step (block Lanczos graphs);
 // sectors with active[s] == 0 are skipped.
-template <int K>
-__global__ void __launch_bounds__(BLOCK, pass_blocks(K))
+template <int K, int BLOCKS, int U>
+__global__ void __launch_bounds__(BLOCK, BLOCKS)
     cache_batch_kernel(const CacheSector* __restrict__ sec, int n_sec, int64_t n_slices,
                        const int64_t* __restrict__ row_off, const void* xv, void* yv, int nvec,
                        const int* __restrict__ x_step, int64_t x_step_elems, const int* __restrict__ active) {
@@ -206,7 +224,7 @@ __global__ void __launch_bounds__(BLOCK, pass_blocks(K))
         const uint32_t* ent = c.ent[ls >> c.chunk_shift] + __ldg(c.boff + ls);
         auto coef = [&](uint32_t w) { return __ldg(ctab + (V::cplx ? 1 : 2) * (w >> ob)); };
         RowSum<K, false> sum;
-        walk<T, AHEAD>(
+        walk<T, U>(
             n, ent, 0u, 255u, lane, [&](uint32_t w) { return x[w & om]; },
             [&](uint32_t w, const T& xj) { sum.add(coef(w), false, xj); });
         if (row >= D) continue;
@@ -217,11 +235,14 @@ __global__ void __launch_bounds__(BLOCK, pass_blocks(K))
     }
 }
 
-template <int K, bool AX, bool DIFF = false, int BLOCKS = pass_blocks(K)>
+template <int K, bool AX, bool DIFF = false, int BLOCKS = pass_blocks(K), int U = AHEAD>
 ed_status launch_pass(const CachePass& p, int sms, cudaStream_t s) {
     if constexpr (K == 1 && BLOCKS != MANY_BLOCKS)
         if (p.mode != 0 && p.n_ent >= MANY_ROW_ENTRIES * (uint64_t)p.D * (uint64_t)p.nb)
             return launch_pass<K, AX, DIFF, MANY_BLOCKS>(p, sms, s);
+    if constexpr (BLOCKS == pass_blocks(K) && U == AHEAD)
+        if (p.mode == 0 && few<K>(p.ns, p.nvec, p.n_ent, p.D, sms))
+            return launch_pass<K, AX, DIFF, few_blocks(K), FEW_AHEAD>(p, sms, s);
     const int64_t need = (p.ns + (BLOCK / 32) - 1) / (BLOCK / 32);
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sms * BLOCKS));
     // the eight-block kernel has no register left for the vector's offset: one launch per vector
@@ -232,8 +253,13 @@ ed_status launch_pass(const CachePass& p, int sms, cudaStream_t s) {
         const dim3 g(grid, (unsigned)together);
         q.x = (const T*)p.x + (int64_t)v * p.D;
         q.y = (T*)p.y + (int64_t)v * p.D;
-        if (p.mode >= 2) cache_pass_kernel<K, AX, true, DIFF, BLOCKS><<<g, BLOCK, 0, s>>>(q);
-        else cache_pass_kernel<K, AX, false, DIFF, BLOCKS><<<g, BLOCK, 0, s>>>(q);
+        if constexpr (U == AHEAD) {
+            if (p.mode >= 2) {
+                cache_pass_kernel<K, AX, true, DIFF, BLOCKS, U><<<g, BLOCK, 0, s>>>(q);
+                continue;
+            }
+        }
+        cache_pass_kernel<K, AX, false, DIFF, BLOCKS, U><<<g, BLOCK, 0, s>>>(q);
     }
     ED_CUDA(cudaGetLastError());
     return ED_OK;
@@ -297,9 +323,16 @@ ed_status cache_batch_launch(const BatchLaunch& L, cudaStream_t s) {
         constexpr int K = decltype(ktag)::value;
         if constexpr (K == 1 || K == 3)
             if (L.nvec > 1 && L.xi) return batch_multi_kind<K>(L, sms, s);
-        const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sms * pass_blocks(K)));
-        cache_batch_kernel<K><<<dim3(grid, (unsigned)L.nvec), BLOCK, 0, s>>>(
-            L.stored, L.n_sec, L.stored_slices, L.row_off, L.x, L.y, L.nvec, L.x_step, L.x_step_elems, L.active);
+        auto launch = [&](auto btag, auto utag) {
+            constexpr int B = decltype(btag)::value;
+            const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sms * B));
+            cache_batch_kernel<K, B, decltype(utag)::value><<<dim3(grid, (unsigned)L.nvec), BLOCK, 0, s>>>(
+                L.stored, L.n_sec, L.stored_slices, L.row_off, L.x, L.y, L.nvec, L.x_step, L.x_step_elems, L.active);
+        };
+        if (few<K>(L.stored_slices, L.nvec, L.stored_entries, L.total_rows, sms))
+            launch(std::integral_constant<int, few_blocks(K)>{}, std::integral_constant<int, FEW_AHEAD>{});
+        else
+            launch(std::integral_constant<int, pass_blocks(K)>{}, std::integral_constant<int, AHEAD>{});
         ED_CUDA(cudaGetLastError());
         return ED_OK;
     };

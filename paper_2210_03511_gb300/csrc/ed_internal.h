@@ -260,6 +260,7 @@ struct BatchLaunch {
     const int* active;         // device [n_sec]: rows of sectors with 0 are skipped (null: all)
     const CacheSector* stored; // device [n_sec]: every sector's stored structure, or null (matrix-free)
     int64_t stored_slices;     // slices of 32 rows over all sectors
+    uint64_t stored_entries;   // and their entries
     void* xi;                  // stored structures, several FP32 vectors: room for their interleaved copy, or null
 };
 ed_status apply_batch_launch(const BatchLaunch& L, cudaStream_t s);
