@@ -703,8 +703,8 @@ ed_status cache_apply(const ed_hamiltonian* h, ed_dtype dt, const void* x, void*
     const size_t copy = cache_interleaved_bytes(dt, nvec, b->dim);
     if (copy) p.xi = h->scratch.get(b->alloc, b->device, copy, s);
     const bool f64 = K == 0 || K == 2;
-    // several warps per slice, interleaved vectors: the general tables
-    const bool ax = K >= 2 && !p.xi && !(nvec == 1 && c.lanes > 1) && (f64 ? c.axis_d : c.axis_f);
+    // several warps per slice: the general tables
+    const bool ax = K >= 2 && !(nvec == 1 && c.lanes > 1) && (f64 ? c.axis_d : c.axis_f);
     const uint8_t* ct = (const uint8_t*)c.ctab.p;
     p.ctab = ct + (f64 ? (ax ? CT_AXD : CT_D2) : (ax ? CT_AXF : CT_F2));
     p.isq = b->dt.blob + (f64 ? b->dt.off_sqrt + (size_t)(b->ht.G + 1) * 8 : b->dt.off_sqrtf + (size_t)(b->ht.G + 1) * 4);

@@ -38,7 +38,7 @@ struct CachePass {
 };
 
 // One segment's pass for p.nvec vectors of kind K, `lanes` warps per slice for
-// one vector.  ax: p.ctab is the axis-aligned table (never with p.xi).
+// one vector.  ax: p.ctab is the axis-aligned table.
 ed_status launch_cache_pass(const CachePass& p, int K, bool ax, int lanes, int sms, cudaStream_t s);
 
 }  // namespace ed

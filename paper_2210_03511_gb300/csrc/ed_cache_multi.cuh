@@ -11,7 +11,8 @@
 // take one-vector passes: they are bound by the FP64 pipe, and the copy won
 // nothing (square32, three vectors: 0.94 against 1.00 ms real, 1.85 against 1.82
 // complex).
-// The sums are those of the one-vector pass, entry by entry.
+// The sums are those of the one-vector pass, entry by entry (complex vectors too: axis-aligned
+// tables where that takes them), so y does not depend on whether there was room for the copy.
 #pragma once
 
 #include <string.h>
@@ -57,16 +58,16 @@ __device__ __forceinline__ void load_part(T (&v)[P], const T* __restrict__ p) {
 }
 
 // The sums of one slice: this lane's part of the rows of its group.
-template <int K, int NV>
+template <int K, int NV, bool AX>
 struct GroupSum {
     using T = typename Val<K>::T;
     using R = typename Val<K>::R;
     using L = Layout<T, NV>;
-    RowSum<K, false> sum[L::G][L::P];
+    RowSum<K, AX> sum[L::G][L::P];
 
     template <typename Coef>
-    __device__ __forceinline__ void run(uint32_t c, const uint32_t* ent, const T* __restrict__ xs, uint32_t ob, int lane,
-                                        Coef&& coef) {
+    __device__ __forceinline__ void run(uint32_t c, const uint32_t* ent, const T* __restrict__ xs, uint32_t ob,
+                                        uint32_t n_re, int lane, Coef&& coef) {
         constexpr int bytes = L::NP * (int)sizeof(T);
         constexpr int ahead = bytes > 16 ? 2 : AHEAD;
         const uint32_t om = (1u << ob) - 1u;
@@ -86,9 +87,10 @@ struct GroupSum {
 #pragma unroll
                 for (int r = 0; r < L::G; ++r) {
                     if (!((has >> (l0 + r)) & 1u)) continue;
-                    const auto cf = coef(x.w[r] >> ob);
+                    const uint32_t cd = x.w[r] >> ob;
+                    const auto cf = coef(cd);
 #pragma unroll
-                    for (int j = 0; j < L::P; ++j) sum[r][j].add(cf, false, x.v[r][j]);
+                    for (int j = 0; j < L::P; ++j) sum[r][j].add(cf, AX && cd >= n_re, x.v[r][j]);
                 }
             });
     }
@@ -128,7 +130,7 @@ __global__ void interleave_kernel(T* __restrict__ xi, const T* __restrict__ x, i
 template <typename T, int NV>
 constexpr int multi_blocks = Layout<T, NV>::NP * sizeof(T) > 32 ? 2 : 4;  // five real vectors 0.58 ms against 0.64 (3)
 
-template <int K, int NV>
+template <int K, int NV, bool AX>
 __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>) cache_pass_multi(CachePass p) {
     using V = Val<K>;
     using T = typename V::T;
@@ -157,7 +159,7 @@ __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>) c
         if (sl + warps < p.ns) nx.load(p, sl + warps, lane);
         const int64_t first = sl * NSLICE + lane - h;  // the group's rows
         bool keep[L::G];                               // whose y is written
-        GroupSum<K, NV> group;
+        GroupSum<K, NV, AX> group;
 #pragma unroll
         for (int r = 0; r < L::G; ++r) {
             const uint32_t cr = L::G == 1 ? c : __shfl_sync(FULL, c, lane - h + r);
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>) c
             for (int j = 0; j < L::P; ++j)
                 if (prev && keep[r] && h * L::P + j < NV) group.sum[r][j].start(y[(int64_t)(h * L::P + j) * D + first + r]);
         }
-        group.run(c, ent, xs, ob, lane, [&](uint32_t cd) { return ctab[cd]; });
+        group.run(c, ent, xs, ob, p.n_re, lane, [&](uint32_t cd) { return ctab[cd]; });
 #pragma unroll
         for (int r = 0; r < L::G; ++r) {
             if (!keep[r]) continue;
@@ -181,7 +183,7 @@ __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>) c
 #pragma unroll
             for (int j = 0; j < L::P; ++j) {
                 if (h * L::P + j >= NV) continue;
-                RowSum<K, false>& sm = group.sum[r][j];
+                RowSum<K, AX>& sm = group.sum[r][j];
                 sm.close();
                 finish<K>(y + (int64_t)(h * L::P + j) * D + row, &xr[j], sm.re, sm.im, last, inv, dg);
             }
@@ -219,8 +221,8 @@ __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>)
         const R* __restrict__ isq;
         if constexpr (K == 0 || K == 2) isq = (const R*)c.sq + c.G1;
         else isq = (const R*)c.sqf + c.G1;
-        GroupSum<K, NV> group;
-        group.run(__ldg(c.counts + row), c.ent[ls >> c.chunk_shift] + __ldg(c.boff + ls), xi, c.off_bits, lane,
+        GroupSum<K, NV, false> group;
+        group.run(__ldg(c.counts + row), c.ent[ls >> c.chunk_shift] + __ldg(c.boff + ls), xi, c.off_bits, 0u, lane,
                [&](uint32_t cd) { return __ldg(ctab + (V::cplx ? 1 : 2) * cd); });
 #pragma unroll
         for (int r = 0; r < L::G; ++r) {
@@ -265,14 +267,19 @@ void launch_interleave(void* xi, const void* x, int64_t total, const int64_t* ro
 }
 
 template <int K>
-ed_status pass_multi_kind(const CachePass& p, int sms, cudaStream_t s) {
+ed_status pass_multi_kind(const CachePass& p, bool ax, int sms, cudaStream_t s) {
     return with_nvec(p.nvec, [&](auto nv) -> ed_status {
         constexpr int NV = decltype(nv)::value;
         if (p.mode < 2) launch_interleave<K, NV>(p.xi, p.x, p.D, nullptr, 1, nullptr, 0, sms, s);
         const int64_t need = (p.ns + (BLOCK / 32) - 1) / (BLOCK / 32);
         const int64_t fit = (int64_t)sms * multi_blocks<typename Val<K>::T, NV>;
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, fit));
-        cache_pass_multi<K, NV><<<grid, BLOCK, 0, s>>>(p);
+        if constexpr (Val<K>::cplx) {
+            if (ax) cache_pass_multi<K, NV, true><<<grid, BLOCK, 0, s>>>(p);
+            else cache_pass_multi<K, NV, false><<<grid, BLOCK, 0, s>>>(p);
+        } else {
+            cache_pass_multi<K, NV, false><<<grid, BLOCK, 0, s>>>(p);
+        }
         ED_CUDA(cudaGetLastError());
         return ED_OK;
     });

@@ -2,6 +2,6 @@
 #include "ed_cache_multi.cuh"
 
 namespace ed {
-template ed_status pass_multi_kind<3>(const CachePass&, int, cudaStream_t);
+template ed_status pass_multi_kind<3>(const CachePass&, bool, int, cudaStream_t);
 template ed_status batch_multi_kind<3>(const BatchLaunch&, int, cudaStream_t);
 }  // namespace ed

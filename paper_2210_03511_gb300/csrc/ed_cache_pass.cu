@@ -19,10 +19,10 @@
 
 namespace ed {
 
-template <int K> ed_status pass_multi_kind(const CachePass& p, int sms, cudaStream_t s);
+template <int K> ed_status pass_multi_kind(const CachePass& p, bool ax, int sms, cudaStream_t s);
 template <int K> ed_status batch_multi_kind(const BatchLaunch& L, int sms, cudaStream_t s);
 #define ED_MULTI(K)                                                                                  \
-    extern template ed_status pass_multi_kind<K>(const CachePass&, int, cudaStream_t);               \
+    extern template ed_status pass_multi_kind<K>(const CachePass&, bool, int, cudaStream_t);              \
     extern template ed_status batch_multi_kind<K>(const BatchLaunch&, int, cudaStream_t);
 ED_MULTI(1) ED_MULTI(3)
 #undef ED_MULTI
@@ -278,7 +278,7 @@ ed_status launch_split(const CachePass& p, int sms, cudaStream_t s) {
 template <int K>
 ed_status launch_kind(const CachePass& p, bool ax, int lanes, int sms, cudaStream_t s) {
     if constexpr (K == 1 || K == 3)
-        if (p.nvec > 1 && p.xi) return pass_multi_kind<K>(p, sms, s);
+        if (p.nvec > 1 && p.xi) return pass_multi_kind<K>(p, ax, sms, s);
     if (lanes > 1 && p.nvec == 1) {
         switch (lanes) {
             case 2: return launch_split<K, 2>(p, sms, s);
