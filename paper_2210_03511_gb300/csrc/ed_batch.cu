@@ -804,7 +804,9 @@ ed_status ed_apply_batch(const ed_batch* B, ed_dtype dtype, const void* x, void*
     BatchLaunch L = make_launch(B, dtype, x, y, nvec);
     if (B->has_sun && !L.stored) return fail(ED_ERR_ARG, "a batch with SU(N) sectors needs every sector's stored structure");
     ED_CUDA(cudaMemsetAsync(B->d_counters.p, 0, 24, (cudaStream_t)stream));
-    const size_t copy = L.stored ? cache_interleaved_bytes(dtype, nvec, B->total) : 0;
+    int sms = 0;
+    ED_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, B->hs[0]->basis->device));
+    const size_t copy = L.stored ? cache_interleaved_bytes(dtype, nvec, B->total, L.stored_slices, sms) : 0;
     if (copy) L.xi = B->scratch.get(*B->alloc, B->hs[0]->basis->device, copy, (cudaStream_t)stream);
     const ed_status st = apply_batch_launch(L, (cudaStream_t)stream);
     if (L.xi) StreamPool::put(L.xi, (cudaStream_t)stream);
@@ -977,8 +979,8 @@ static ed_status block_lanczos(const ed_batch* B, const ed_block_lanczos_opts* o
     L.active = active;
     L.x_step = dk;
     L.x_step_elems = bs;
-    const size_t copy = L.stored ? cache_interleaved_bytes(o->dtype, b, tot) : 0;
-    if (copy) L.xi = get(copy);  // without it: one vector after another
+    const size_t copy = L.stored ? cache_interleaved_bytes(o->dtype, b, tot, L.stored_slices, sms) : 0;
+    if (copy) L.xi = get(copy);  // without it: the one-vector passes
     auto step = [&]() -> ed_status {
         ed_status st = apply_batch_launch(L, s);  // W = H V_k
         if (st != ED_OK) return st;

@@ -700,7 +700,7 @@ ed_status cache_apply(const ed_hamiltonian* h, ed_dtype dt, const void* x, void*
     p.off_bits = (uint32_t)c.off_bits;
     p.n_re = (uint32_t)c.n_re;
     const int K = dt == ED_F64 ? 0 : dt == ED_F32 ? 1 : dt == ED_C128 ? 2 : 3;
-    const size_t copy = cache_interleaved_bytes(dt, nvec, b->dim);
+    const size_t copy = cache_interleaved_bytes(dt, nvec, b->dim, c.ns, c.sms);
     if (copy) p.xi = h->scratch.get(b->alloc, b->device, copy, s);
     const bool f64 = K == 0 || K == 2;
     // several warps per slice: the general tables

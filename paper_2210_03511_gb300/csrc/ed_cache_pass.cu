@@ -309,8 +309,18 @@ ed_status launch_cache_pass(const CachePass& p, int K, bool ax, int lanes, int s
     return fail(ED_ERR_ARG, "bad value kind");
 }
 
-size_t cache_interleaved_bytes(ed_dtype dt, int nvec, int64_t rows) {
+// Several FP32 vectors are copied unless the blocks of all their one-vector passes are
+// resident at once: side by side these then take about as long as one, without scratch
+// (whose pool takes 0.1 ms to make on an owner's first call) and without a launch for
+// the copy.  triangular24 (28,699 rows, 112 blocks a vector), five vectors: real 35 -> 18 us,
+// complex 38 -> 25 us; square16 (153 rows) 20.6 -> 8.3 us.  Just above the line the copy is
+// as good or better: 56,682 rows of triangular24, four complex vectors 44 us side by side
+// against 35, two complex ones of square26 (784 blocks) 36 against 27, two real ones 23
+// against 25.
+size_t cache_interleaved_bytes(ed_dtype dt, int nvec, int64_t rows, int64_t slices, int sms) {
     if (nvec < 2 || dt == ED_F64 || dt == ED_C128) return 0;
+    const int K = dt == ED_F32 ? 1 : 3;
+    if ((slices + (BLOCK / 32) - 1) / (BLOCK / 32) * nvec <= (int64_t)sms * pass_blocks(K)) return 0;
     return (size_t)(nvec <= 2 ? 2 : (nvec <= 4 ? 4 : 8)) * (size_t)rows * (dt == ED_F32 ? 4 : 8);
 }
 

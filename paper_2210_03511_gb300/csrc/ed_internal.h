@@ -267,8 +267,8 @@ ed_status apply_batch_launch(const BatchLaunch& L, cudaStream_t s);
 // the batched stored-structure H.x (ed_cache_pass.cu), and the descriptor of
 // one Hamiltonian's structure (ed_cache.cu; false unless stored in one segment)
 ed_status cache_batch_launch(const BatchLaunch& L, cudaStream_t s);
-// bytes of the interleaved copy of nvec vectors of `rows` rows (0: none is made)
-size_t cache_interleaved_bytes(ed_dtype dt, int nvec, int64_t rows);
+// bytes of the interleaved copy of nvec vectors of `rows` rows in `slices` slices (0: none is made)
+size_t cache_interleaved_bytes(ed_dtype dt, int nvec, int64_t rows, int64_t slices, int sms);
 bool cache_sector_desc(const ed_hamiltonian* h, CacheSector& d);
 size_t hx_smem_bytes(const ed_hamiltonian* h, ed_dtype dt, bool ns_ok, int nvec, int blocks);
 int hx_default_blocks(const ed_hamiltonian* h, ed_dtype dt, bool ns_ok, int nvec);
