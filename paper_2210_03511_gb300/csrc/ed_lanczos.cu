@@ -426,12 +426,20 @@ __global__ void __launch_bounds__(256) multi_axpy_kernel(typename LV<K>::T* w, c
 }
 
 // Two elements a thread where the grid does not cover the vector anyway (a second
-// one that repeats the first would double the FP64 work of a small sector).
+// one that repeats the first would double the FP64 work of a small sector).  Complex
+// vector by vector sums (DIFF) take one: their two chains of dependent operations per
+// element are long enough, and two elements were slower (338,376 rows, mean of 1 to 30
+// stored vectors: 37.5 us with one, 62.8 with two).
 template <int K, bool DIFF = false>
 static void multi_axpy(typename LV<K>::T* w, const typename LV<K>::T* A, int64_t ld, int nk, const double2* c, int64_t n,
                        unsigned g, cudaStream_t s) {
-    if (n > (int64_t)g * 256) multi_axpy_kernel<K, DIFF, 2><<<g, 256, 0, s>>>(w, A, ld, nk, c, n);
-    else multi_axpy_kernel<K, DIFF, 1><<<g, 256, 0, s>>>(w, A, ld, nk, c, n);
+    if constexpr (!(LV<K>::cplx && DIFF)) {
+        if (n > (int64_t)g * 256) {
+            multi_axpy_kernel<K, DIFF, 2><<<g, 256, 0, s>>>(w, A, ld, nk, c, n);
+            return;
+        }
+    }
+    multi_axpy_kernel<K, DIFF, 1><<<g, 256, 0, s>>>(w, A, ld, nk, c, n);
 }
 
 // out = sum_k s_k A_k with real coefficients s (FP64 accumulation, output type O)
