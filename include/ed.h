@@ -327,8 +327,9 @@ ed_status ed_apply(const ed_hamiltonian* h, ed_dtype dtype, const void* x, void*
  * ED_ERR_NOMEM is returned (ed_apply stays matrix-free).  Also
  * ED_ERR_TABLE_TOO_LARGE when more than 256 distinct coefficients occur,
  * ED_ERR_ARG for more than 255 flip terms.  The build takes scratch from the
- * same allocator (8 bytes per flip term for a chunk of rows, up to about 3 GB;
- * 64 MB when the allocator has no room for that), released on return.
+ * same allocator (8 bytes per flip term and row for a chunk of rows, up to
+ * about 3 GB; less when the allocator has no room for that, down to a few per
+ * cent of the structure), released on return.
  * Synchronous on `stream`.
  * A second call replaces the stored structure. */
 ed_status ed_hamiltonian_store(ed_hamiltonian* h, ed_dtype dtype, int32_t seg_log2, size_t max_bytes,

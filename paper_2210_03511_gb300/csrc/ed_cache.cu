@@ -465,30 +465,31 @@ struct Codes {
 
 // Builds the structure into h->cache, its chunks' scratch limited to about
 // `scratch` bytes.  On an error the parts stay in h->cache for cache_free;
-// over_limit: whether it was max_bytes that stopped it.
+// smaller: the scratch of another try, where the memory had no room for this one's
+// and less scratch may make some (0: it may not).
 static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_t scratch, Codes& codes,
-                            cudaStream_t s, bool& over_limit) {
+                            cudaStream_t s, size_t& smaller) {
     const ed_basis* b = h->basis;
     const HostTables& t = b->ht;
     const Alloc& A = b->alloc;
     const int64_t D = b->dim;
     const int nb = (int)(((uint64_t)D + ((uint64_t)1 << bits) - 1) >> bits);
     HCache& c = h->cache;
-    over_limit = false;
+    smaller = 0;
     BuildScratch sc{&A, s, {}};
     c.seg_bits = bits;
     c.nb = nb;
     c.ns = (D + NSLICE - 1) / NSLICE;
     c.off_bits = std::max(24, bits);
     const int64_t ns = c.ns, Dpad = ns * NSLICE;
-    // chunk: a power of two of rows whose raw entries fit the scratch
+    // chunk: a power of two of rows whose raw entries fit the scratch; the only chunk: all rows
     const int64_t row_bytes = 8 * (int64_t)std::max(h->n_flip, 1) + 1;
-    int64_t R = 1 << 12;
-    while (R * 2 * row_bytes <= (int64_t)scratch && R < (1 << 22) && R < Dpad) R *= 2;
+    int64_t chunk = NSLICE;
+    while (chunk * 2 * row_bytes <= (int64_t)scratch && chunk < (1 << 22) && chunk < Dpad) chunk *= 2;
     c.chunk_shift = 0;
-    while (((int64_t)NSLICE << c.chunk_shift) < R) ++c.chunk_shift;
-    const int64_t n_chunks = (Dpad + R - 1) / R;
-    const int64_t Rsl = R / NSLICE;
+    while (((int64_t)NSLICE << c.chunk_shift) < chunk) ++c.chunk_shift;
+    const int64_t n_chunks = (Dpad + chunk - 1) / chunk;
+    const int64_t R = std::min(chunk, Dpad), Rsl = R / NSLICE;
     codes.reset(1 << (32 - c.off_bits));
     auto get = [&](DevBuf& d, size_t bytes) {
         d.bytes = bytes;
@@ -521,8 +522,10 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
     uint32_t* d_tot = (uint32_t*)(scr + o_tot);
     uint64_t* d_abs = (uint64_t*)(scr + o_abs);
     uint64_t* d_tiles = (uint64_t*)(scr + o_tiles);
-    if (!ok || !scr)
+    if (!ok || !scr) {
+        if (ok && chunk > NSLICE) smaller = std::min(scratch, at) / 32;
         return fail(ED_ERR_NOMEM, "structure build: allocation failed");
+    }
     ED_CUDA(cudaMemcpyAsync(d_hmap, codes.hmap.data(), codes.hmap.size() * 2, cudaMemcpyHostToDevice, s));
     ED_CUDA(cudaMemcpyAsync(d_chi, codes.chi_id.data(), codes.chi_id.size() * 2, cudaMemcpyHostToDevice, s));
     ED_CUDA(cudaMemsetAsync(d_cnt, 0, o_code - o_cnt, s));  // counters and seen bits
@@ -555,8 +558,8 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
     std::vector<uint64_t> base((size_t)n_chunks, 0);
     unsigned long long cnt[4] = {};
     for (int64_t k = 0; k < n_chunks; ++k) {
-        q.r0 = k * R;
-        q.r1 = std::min<int64_t>(q.r0 + R, Dpad);
+        q.r0 = k * chunk;
+        q.r1 = std::min<int64_t>(q.r0 + chunk, Dpad);
         ed_status st = search_dispatch(q, smem, t.n_sub, ns_ok, w8, ch, s);
         if (st != ED_OK) return st;
         const int64_t nsl = (q.r1 - q.r0) / NSLICE, n = nsl * nb;
@@ -589,13 +592,14 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
         DevBuf e;
         e.bytes = (size_t)edge[nb] * 4 + 16;
         need += (size_t)edge[nb] * 4 + (k == 0 ? 16 : 0);
-        if (need > max_bytes) {
-            over_limit = true;
+        if (need > max_bytes)
             return fail(ED_ERR_NOMEM, "the stored structure needs %zu bytes or more, over the limit of %zu", need,
                         max_bytes);
-        }
         e.p = A.get(e.bytes, s);
-        if (!e.p) return fail(ED_ERR_NOMEM, "structure entries (%zu bytes)", e.bytes);
+        if (!e.p) {
+            if (chunk > NSLICE && at > need / 32) smaller = std::min(scratch, at) / 32;
+            return fail(ED_ERR_NOMEM, "structure entries (%zu bytes)", e.bytes);
+        }
         c.ent.push_back(e);
         base[k] = (uint64_t)(uintptr_t)e.p;
         CachePack pk{};
@@ -665,12 +669,14 @@ ed_status cache_build(ed_hamiltonian* h, ed_dtype dtype, int seg_log2, size_t ma
     codes.init(h);
     if (codes.n_keys > ((uint64_t)1 << 26))
         return fail(ED_ERR_TABLE_TOO_LARGE, "coefficient key space of %llu too large", (unsigned long long)codes.n_keys);
-    // about 3 GB of scratch, or 64 MB where the memory has no room for that
-    bool over_limit = false;
-    ed_status st = build_once(h, bits, max_bytes, (size_t)3 << 30, codes, s, over_limit);
-    if (st == ED_ERR_NOMEM && !over_limit) {
+    // about 3 GB of scratch, and less and less where the memory has no room for that beside the
+    // structure, until the scratch is not what is in the way (a few per cent of the structure)
+    size_t scratch = (size_t)3 << 30;
+    ed_status st = build_once(h, bits, max_bytes, scratch, codes, s, scratch);
+    while (st == ED_ERR_NOMEM && scratch) {
+        cudaStreamSynchronize(s);
         cache_free(h);
-        st = build_once(h, bits, max_bytes, (size_t)64 << 20, codes, s, over_limit);
+        st = build_once(h, bits, max_bytes, scratch, codes, s, scratch);
     }
     if (st != ED_OK) {
         cudaStreamSynchronize(s);  // nothing may still write into what is freed
