@@ -590,8 +590,8 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
         }
         c.n_ent += edge[nb];
         DevBuf e;
-        e.bytes = (size_t)edge[nb] * 4 + 16;
-        need += (size_t)edge[nb] * 4 + (k == 0 ? 16 : 0);
+        e.bytes = std::max<size_t>((size_t)edge[nb] * 4, 16);
+        need += e.bytes;
         if (need > max_bytes)
             return fail(ED_ERR_NOMEM, "the stored structure needs %zu bytes or more, over the limit of %zu", need,
                         max_bytes);
