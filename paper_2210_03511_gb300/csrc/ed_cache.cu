@@ -30,7 +30,8 @@
 // count up from 0, the others down from the largest code).
 //
 // Build.  Rows are taken in chunks: one search pass writes every entry of the
-// chunk as (column, coefficient key) to scratch and counts entries per row and
+// chunk as (column, coefficient key) to scratch (in one word of 32 bits where both
+// fit) and counts entries per row and
 // segment; the slices' offsets are scanned, the chunk's entries allocated and
 // packed.  Searching costs far more than the 16 bytes of scratch traffic per
 // entry, so one search and a pack (36-site kagome sector, 4.7 10^9 entries: 159
@@ -53,7 +54,8 @@ struct CacheSearch {
     HxArgs a;                      // basis and terms (x, y unused)
     int seg_bits, nb;
     int64_t r0, r1, R;             // rows of the chunk, its scratch stride
-    uint2* raw;                    // [n_flip][R] (column, key) of the row's k-th entry
+    void* raw;                     // [n_flip][R] (column, key) of the row's k-th entry: uint2, or
+    int key_shift;                 // one word, key << key_shift | column, when key_shift > 0
     uint8_t* rowtot;               // [R] entries of the row
     uint8_t* counts;               // [nb][Dpad] entries of the row per segment
     int64_t Dpad;
@@ -182,7 +184,9 @@ __global__ void __launch_bounds__(BLOCK, hx_min_blocks(sizeof(W), 1, 0)) cache_s
                 ++cnt[(uint64_t)jx >> c.seg_bits];
                 const uint32_t bit = 1u << (key & 31);
                 if (!(c.seen[key >> 5] & bit)) atomicOr(&c.seen[key >> 5], bit);
-                c.raw[(int64_t)k * c.R + r] = make_uint2((uint32_t)jx, key);
+                if (sizeof(W) == 4 && c.key_shift)
+                    ((uint32_t*)c.raw)[(int64_t)k * c.R + r] = key << c.key_shift | (uint32_t)jx;
+                else ((uint2*)c.raw)[(int64_t)k * c.R + r] = make_uint2((uint32_t)jx, key);
                 ++k;
             }
         }
@@ -228,7 +232,8 @@ __global__ void slice_offsets(const uint64_t* abs_off, int64_t nsl, int nb, int6
 struct CachePack {
     int seg_bits, nb, off_bits;
     int64_t r0, r1, R, Dpad, ns;
-    const uint2* raw;              // [n_flip][R]
+    const void* raw;               // [n_flip][R], as CacheSearch
+    int key_shift;
     const uint8_t* rowtot;         // [R]
     const uint8_t* counts;         // [nb][Dpad]
     const uint32_t* boff;          // [nb][ns]
@@ -242,7 +247,16 @@ struct CachePack {
 // lanes i < l and min(c_i, k) of the others (c_i: the lanes' counts in the
 // segment, four to a word).  With one segment all lanes are at the same k and a
 // ballot gives the place.
+template <bool WORD, bool ONE>  // entries of one word; one segment
 __global__ void __launch_bounds__(BLOCK) cache_pack_kernel(CachePack a) {
+    auto load = [&](int64_t at) -> uint2 {
+        if constexpr (WORD) {
+            const uint32_t w = __ldg((const uint32_t*)a.raw + at);
+            return make_uint2(w & ((1u << a.key_shift) - 1u), w >> a.key_shift);
+        } else {
+            return __ldg((const uint2*)a.raw + at);
+        }
+    };
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t segmask = (uint32_t)(((uint64_t)1 << a.seg_bits) - 1);
@@ -259,38 +273,47 @@ __global__ void __launch_bounds__(BLOCK) cache_pack_kernel(CachePack a) {
          sl < a.r1 / NSLICE; sl += warps) {
         const int64_t row = sl * NSLICE + lane, r = row - a.r0;
         const int n = a.rowtot[r];
-        if (a.nb == 1) {
+        if constexpr (ONE) {
             uint32_t* out = a.ent + a.boff[sl];
             const int m = __reduce_max_sync(0xffffffffu, n);
-            for (int k = 0; k < m; ++k) {
-                const unsigned has = __ballot_sync(0xffffffffu, n > k);
-                if (n > k) {
-                    const uint2 e = a.raw[(int64_t)k * a.R + r];
-                    out[__popc(has & lt)] = ((uint32_t)__ldg(a.code + e.y) << a.off_bits) | e.x;
-                }
-                out += __popc(has);
-            }
-            continue;
-        }
-        for (int b = 0; b < a.nb; ++b) kb[b] = 0;
-        for (int i = 0; i < n; ++i) {
-            const uint2 e = a.raw[(int64_t)i * a.R + r];
-            const int b = (int)(e.x >> a.seg_bits);
-            const uint32_t k = kb[b];
-            kb[b] = (uint8_t)(k + 1);
-            const uint4* cw = (const uint4*)(a.counts + (int64_t)b * a.Dpad + sl * NSLICE);
-            const uint4 lo = cw[0], hi = cw[1];
-            const uint32_t c[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-            const uint32_t kk = k * 0x01010101u;
-            uint32_t o = 0;
+            constexpr int U = 4;  // entries in flight: a slice is one chain of entry and code loads (0.01 ms of 0.3)
+            for (int k = 0; k < m; k += U) {
+                uint2 e[U];
+                uint32_t w[U];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) o += __vsadu4(__vminu4(c[q], kk + before[q]), 0u);
-            if (k >= ((const uint8_t*)cw)[lane]) {
-                ++over;
-                continue;
+                for (int u = 0; u < U; ++u)
+                    if (n > k + u) e[u] = load((int64_t)(k + u) * a.R + r);
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (n > k + u) w[u] = ((uint32_t)__ldg(a.code + e[u].y) << a.off_bits) | e[u].x;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const unsigned has = __ballot_sync(0xffffffffu, n > k + u);
+                    if (n > k + u) out[__popc(has & lt)] = w[u];
+                    out += __popc(has);
+                }
             }
-            a.ent[(int64_t)a.boff[(int64_t)b * a.ns + sl] + o] =
-                ((uint32_t)__ldg(a.code + e.y) << a.off_bits) | (e.x & segmask);
+        } else {
+            for (int b = 0; b < a.nb; ++b) kb[b] = 0;
+            for (int i = 0; i < n; ++i) {
+                const uint2 e = load((int64_t)i * a.R + r);
+                const int b = (int)(e.x >> a.seg_bits);
+                const uint32_t k = kb[b];
+                kb[b] = (uint8_t)(k + 1);
+                const uint4* cw = (const uint4*)(a.counts + (int64_t)b * a.Dpad + sl * NSLICE);
+                const uint4 lo = cw[0], hi = cw[1];
+                const uint32_t c[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+                const uint32_t kk = k * 0x01010101u;
+                uint32_t o = 0;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) o += __vsadu4(__vminu4(c[q], kk + before[q]), 0u);
+                if (k >= ((const uint8_t*)cw)[lane]) {
+                    ++over;
+                    continue;
+                }
+                a.ent[(int64_t)a.boff[(int64_t)b * a.ns + sl] + o] =
+                    ((uint32_t)__ldg(a.code + e.y) << a.off_bits) | (e.x & segmask);
+            }
         }
     }
     if (over) atomicAdd(a.counters + 3, over);
@@ -482,8 +505,20 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
     c.ns = (D + NSLICE - 1) / NSLICE;
     c.off_bits = std::max(24, bits);
     const int64_t ns = c.ns, Dpad = ns * NSLICE;
-    // chunk: a power of two of rows whose raw entries fit the scratch; the only chunk: all rows
-    const int64_t row_bytes = 8 * (int64_t)std::max(h->n_flip, 1) + 1;
+    // chunk: a power of two of rows whose raw entries fit the scratch; the only chunk: all rows.
+    // Column and key in one word where they fit (32-bit states; sectors of 64-bit states are large,
+    // and the choice cost their search 4 %, square36 219 -> 229 ms): an allocation that needs 2 MB
+    // of its own costs as much as the build of a small sector (chain16, 12,870 rows: 0.30 ms with
+    // two words, 0.16 with one; square32 7.0 -> 5.8 ms)
+    auto width = [](uint64_t n) {
+        int k = 1;
+        while (((uint64_t)1 << k) < n) ++k;
+        return k;
+    };
+    const int col_bits = width((uint64_t)D);
+    const int key_shift = b->word == 4 && col_bits + width(codes.n_keys) <= 32 ? col_bits : 0;
+    const size_t raw_bytes = key_shift ? sizeof(uint32_t) : sizeof(uint2);
+    const int64_t row_bytes = (int64_t)raw_bytes * std::max(h->n_flip, 1) + 1;
     int64_t chunk = NSLICE;
     while (chunk * 2 * row_bytes <= (int64_t)scratch && chunk < (1 << 22) && chunk < Dpad) chunk *= 2;
     c.chunk_shift = 0;
@@ -508,7 +543,7 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
     };
     const size_t o_hmap = part(codes.hmap.size() * 2), o_chi = part(codes.chi_id.size() * 2), o_cnt = part(64),
                  o_seen = part(seen_bytes), o_code = part((size_t)codes.n_keys),
-                 o_raw = part((size_t)std::max(h->n_flip, 1) * R * sizeof(uint2)), o_tot1 = part((size_t)R),
+                 o_raw = part((size_t)std::max(h->n_flip, 1) * R * raw_bytes), o_tot1 = part((size_t)R),
                  o_tot = part((size_t)nb * Rsl * 4), o_abs = part(((size_t)nb * Rsl + 1) * 8),
                  o_tiles = part(scan_scratch_words((uint64_t)nb * Rsl) * 8);
     uint8_t* scr = (uint8_t*)sc.get(at);
@@ -517,7 +552,7 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
     unsigned long long* d_cnt = (unsigned long long*)(scr + o_cnt);
     uint32_t* d_seen = (uint32_t*)(scr + o_seen);
     uint8_t* d_code = scr + o_code;
-    uint2* d_raw = (uint2*)(scr + o_raw);
+    void* d_raw = scr + o_raw;
     uint8_t* d_rowtot = scr + o_tot1;
     uint32_t* d_tot = (uint32_t*)(scr + o_tot);
     uint64_t* d_abs = (uint64_t*)(scr + o_abs);
@@ -536,6 +571,7 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
     q.nb = nb;
     q.R = R;
     q.raw = d_raw;
+    q.key_shift = key_shift;
     q.rowtot = d_rowtot;
     q.counts = (uint8_t*)c.counts.p;
     q.Dpad = Dpad;
@@ -612,13 +648,17 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
         pk.Dpad = Dpad;
         pk.ns = ns;
         pk.raw = d_raw;
+        pk.key_shift = key_shift;
         pk.rowtot = d_rowtot;
         pk.counts = q.counts;
         pk.boff = (const uint32_t*)c.boff.p;
         pk.code = d_code;
         pk.ent = (uint32_t*)e.p;
         pk.counters = d_cnt;
-        cache_pack_kernel<<<(unsigned)std::min<int64_t>((nsl + 7) / 8, (int64_t)c.sms * 8), BLOCK, 0, s>>>(pk);
+        const unsigned pg = (unsigned)std::min<int64_t>((nsl + 7) / 8, (int64_t)c.sms * 8);
+        auto pack = key_shift ? (nb == 1 ? cache_pack_kernel<true, true> : cache_pack_kernel<true, false>)
+                              : (nb == 1 ? cache_pack_kernel<false, true> : cache_pack_kernel<false, false>);
+        pack<<<pg, BLOCK, 0, s>>>(pk);
         ED_CUDA(cudaGetLastError());
     }
     // coefficient tables; axis-aligned ones: (c, c) for a real c, (-c, c) for i c
