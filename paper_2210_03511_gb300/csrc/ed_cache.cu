@@ -417,6 +417,7 @@ struct Codes {
     uint64_t G1 = 0, n_keys = 0;
     std::vector<uint32_t> seen;      // keys that have a code
     std::vector<uint8_t> code;
+    std::vector<double> d1;          // [NCODE] coefficients of real Hamiltonians, FP64
     std::vector<double> d2;          // [NCODE][2] coefficients, FP64
     std::vector<float> f2;           // and FP32
     int cap = NCODE, n_re = 0, n_im = 0;
@@ -452,6 +453,7 @@ struct Codes {
         n_re = n_im = 0;
         seen.assign((n_keys + 31) / 32, 0u);
         code.assign((size_t)n_keys, 0);
+        d1.assign(NCODE, 0.0);
         d2.assign(2 * NCODE, 0.0);
         f2.assign(2 * NCODE, 0.f);
     }
@@ -467,11 +469,13 @@ struct Codes {
                 const auto& cv = cval[hc % cval.size()];
                 const auto& hv = hval[hc / cval.size()];
                 // conj(h) chi sqrt(n), h = jhalf + i him: the matrix-free kernel's coefficient of
-                // this gather in each precision (real kinds: its real part)
+                // this gather in each precision (real FP32: its real part; real FP64: jhalf sqrt(n)
+                // with the sign of chi, which may differ from -1 and 1 by rounding)
                 const double sq = sqrt((double)nst);
                 const double re = (hv.first * cv.first + hv.second * cv.second) * sq;
                 const double im = (hv.first * cv.second - hv.second * cv.first) * sq;
                 const int id = im == 0.0 ? n_re++ : cap - 1 - n_im++;
+                d1[id] = cv.first < 0.0 ? -(hv.first * sq) : hv.first * sq;
                 d2[2 * id] = re;
                 d2[2 * id + 1] = im;
                 const float jf = (float)hv.first, hf = (float)hv.second, cx = (float)cv.first, cy = (float)cv.second;
@@ -681,6 +685,7 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
     }
     uint8_t* ct = (uint8_t*)c.ctab.p;
     ED_CUDA(cudaMemcpyAsync(ct + CT_D2, codes.d2.data(), NCODE * 16, cudaMemcpyHostToDevice, s));
+    ED_CUDA(cudaMemcpyAsync(ct + CT_D1, codes.d1.data(), NCODE * 8, cudaMemcpyHostToDevice, s));
     ED_CUDA(cudaMemcpyAsync(ct + CT_F2, codes.f2.data(), NCODE * 8, cudaMemcpyHostToDevice, s));
     ED_CUDA(cudaMemcpyAsync(ct + CT_AXD, a_d2.data(), NCODE * 16, cudaMemcpyHostToDevice, s));
     ED_CUDA(cudaMemcpyAsync(ct + CT_AXF, a_f2.data(), NCODE * 8, cudaMemcpyHostToDevice, s));
@@ -752,7 +757,7 @@ ed_status cache_apply(const ed_hamiltonian* h, ed_dtype dt, const void* x, void*
     // several warps per slice: the general tables
     const bool ax = K >= 2 && !(nvec == 1 && c.lanes > 1) && (f64 ? c.axis_d : c.axis_f);
     const uint8_t* ct = (const uint8_t*)c.ctab.p;
-    p.ctab = ct + (f64 ? (ax ? CT_AXD : CT_D2) : (ax ? CT_AXF : CT_F2));
+    p.ctab = ct + (ax ? (f64 ? CT_AXD : CT_AXF) : K == 0 ? CT_D1 : K == 2 ? CT_D2 : CT_F2);
     p.isq = b->dt.blob + (f64 ? b->dt.off_sqrt + (size_t)(b->ht.G + 1) * 8 : b->dt.off_sqrtf + (size_t)(b->ht.G + 1) * 4);
     ed_status st = ED_OK;
     for (int k = 0; k < c.nb && st == ED_OK; ++k) {

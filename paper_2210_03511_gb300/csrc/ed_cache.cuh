@@ -9,10 +9,17 @@ namespace ed {
 constexpr int NCODE = 256;    // coefficient codes at most (one byte)
 constexpr int NSLICE = 32;    // rows of a slice (one warp)
 
-// Byte offsets of the tables in HCache::ctab (a real coefficient is the real
-// part of the complex one).
+// Byte offsets of the tables in HCache::ctab.  A real FP32 coefficient is the real part of
+// the complex one; a real FP64 one has its own table (the character enters as its sign,
+// as in the matrix-free kernel, whose bits the real sums keep).
 constexpr size_t CT_D2 = 0, CT_F2 = (size_t)NCODE * 16, CT_AXD = (size_t)NCODE * 24, CT_AXF = (size_t)NCODE * 40,
-                 CT_BYTES = (size_t)NCODE * 48;
+                 CT_D1 = (size_t)NCODE * 48, CT_BYTES = (size_t)NCODE * 56;
+
+// Coefficient of code 0 of a kind, and the step from code to code in coefficients of the kind.
+template <int K>
+constexpr size_t ct_offset = K == 0 ? CT_D1 : (K == 2 ? CT_D2 : CT_F2);
+template <int K>
+constexpr int ct_step = K == 1 ? 2 : 1;
 
 // Arguments of one segment's pass of the stored-structure H.x.
 struct CachePass {
@@ -22,7 +29,7 @@ struct CachePass {
     const void* x;              // [nvec][D]
     void* xi;                   // several FP32 vectors: room for their copy interleaved by row (filled at mode 0 and 1), or null
     void* y;                    // [nvec][D]
-    const void* ctab;           // [256] complex coefficients of the value kind's precision
+    const void* ctab;           // coefficients: ct_offset<K>, or an axis-aligned table
     const void* isq;            // [G+1] 1/sqrt(k) of the value kind's real type
     const uint16_t* stab;       // [D] |Stab sigma_i|
     const double* diag;         // [D] Ising part

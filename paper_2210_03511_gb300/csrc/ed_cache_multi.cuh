@@ -217,13 +217,13 @@ __global__ void __launch_bounds__(BLOCK, multi_blocks<typename Val<K>::T, NV>)
         const int64_t ls = gs - c.slice0, D = c.D, row = ls * NSLICE + lane;
         const T* __restrict__ xi = (const T*)xiv + row_off[lo] * NP;
         T* __restrict__ y = (T*)yv + (int64_t)NV * row_off[lo];
-        const CT* __restrict__ ctab = (const CT*)(c.ctab + (K == 0 || K == 2 ? CT_D2 : CT_F2));
+        const CT* __restrict__ ctab = (const CT*)(c.ctab + ct_offset<K>);
         const R* __restrict__ isq;
         if constexpr (K == 0 || K == 2) isq = (const R*)c.sq + c.G1;
         else isq = (const R*)c.sqf + c.G1;
         GroupSum<K, NV, false> group;
         group.run(__ldg(c.counts + row), c.ent[ls >> c.chunk_shift] + __ldg(c.boff + ls), xi, c.off_bits, 0u, lane,
-               [&](uint32_t cd) { return __ldg(ctab + (V::cplx ? 1 : 2) * cd); });
+               [&](uint32_t cd) { return __ldg(ctab + ct_step<K> * cd); });
 #pragma unroll
         for (int r = 0; r < L::G; ++r) {
             const int64_t at = row - h + r;

@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCKS)
         const int64_t ls = gs - c.slice0, D = c.D;
         const T* __restrict__ x = xb + (int64_t)nvec * row_off[lo] + (int64_t)blockIdx.y * D;
         T* __restrict__ y = yb + (int64_t)nvec * row_off[lo] + (int64_t)blockIdx.y * D;
-        const CT* __restrict__ ctab = (const CT*)(c.ctab + (K == 0 || K == 2 ? CT_D2 : CT_F2));
+        const CT* __restrict__ ctab = (const CT*)(c.ctab + ct_offset<K>);
         const R* __restrict__ isq;
         if constexpr (K == 0 || K == 2) isq = (const R*)c.sq + c.G1;
         else isq = (const R*)c.sqf + c.G1;
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCKS)
         const int64_t row = ls * NSLICE + lane;
         const uint32_t n = __ldg(c.counts + row);
         const uint32_t* ent = c.ent[ls >> c.chunk_shift] + __ldg(c.boff + ls);
-        auto coef = [&](uint32_t w) { return __ldg(ctab + (V::cplx ? 1 : 2) * (w >> ob)); };
+        auto coef = [&](uint32_t w) { return __ldg(ctab + ct_step<K> * (w >> ob)); };
         RowSum<K, false> sum;
         walk<T, U>(
             n, ent, 0u, 255u, lane, [&](uint32_t w) { return x[w & om]; },

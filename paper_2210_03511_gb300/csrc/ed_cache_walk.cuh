@@ -146,8 +146,7 @@ __device__ __forceinline__ void finish(typename Val<K>::T* y, const typename Val
 template <int K, typename CT>
 __device__ __forceinline__ void stage_codes(CT* dst, const void* src) {
     for (int i = threadIdx.x; i < NCODE; i += blockDim.x) {
-        if constexpr (Val<K>::cplx) dst[i] = ((const CT*)src)[i];
-        else dst[i] = ((const CT*)src)[2 * i];  // real part of the complex table
+        dst[i] = ((const CT*)src)[ct_step<K> * i];
     }
 }
 
