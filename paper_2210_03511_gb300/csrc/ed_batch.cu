@@ -1255,6 +1255,12 @@ static ed_status block_lanczos(const ed_batch* B, const ed_block_lanczos_opts* o
             for (auto& th : pool) th.join();
         }
         for (int sct = 0; sct < n; ++sct) its_last[sct] = std::max(1, its_last[sct]);
+        if (L.xi) {  // the steps are over: room for the refinement's vectors
+            ED_CUDA(cudaStreamSynchronize(s));
+            A.put(L.xi, copy, 0);
+            bufs.erase(std::find(bufs.begin(), bufs.end(), std::make_pair(L.xi, copy)));
+            L.xi = nullptr;
+        }
         double2* Zd = (double2*)get(Zh.size() * sizeof(double2));
         int* its_d = (int*)get((size_t)n * 4);
         int* act_all = (int*)get((size_t)n * 4);
