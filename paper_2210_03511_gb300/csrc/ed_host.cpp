@@ -44,17 +44,44 @@ void* Alloc::get(size_t bytes, cudaStream_t s) const {
     if (bytes == 0) bytes = 16;
     if (custom) return a.alloc(bytes, (ed_stream)s, a.ctx);
     void* p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    for (bool again = true;; again = false) {
+        const cudaError_t e = cudaMalloc(&p, bytes);
+        if (e == cudaSuccess) return p;
         cudaGetLastError();
-        return nullptr;
+        if (!again || e != cudaErrorMemoryAllocation || !StreamPool::trim()) return nullptr;
     }
-    return p;
 }
 
 void Alloc::put(void* p, size_t bytes, cudaStream_t s) const {
     if (!p) return;
     if (custom) a.free(p, bytes, (ed_stream)s, a.ctx);
     else cudaFree(p);
+}
+
+// The pools that exist.  Never destroyed: owners may be freed at any time before exit.
+struct Pools {
+    std::mutex mu;
+    std::vector<cudaMemPool_t> list;
+    static Pools& all() {
+        static Pools* p = new Pools;
+        return *p;
+    }
+};
+
+bool StreamPool::trim() {
+    Pools& all = Pools::all();
+    std::lock_guard<std::mutex> l(all.mu);
+    for (cudaMemPool_t p : all.list) cudaMemPoolTrimTo(p, 0);
+    cudaGetLastError();
+    return !all.list.empty();
+}
+
+StreamPool::~StreamPool() {
+    if (!pool) return;
+    Pools& all = Pools::all();
+    std::lock_guard<std::mutex> l(all.mu);
+    all.list.erase(std::find(all.list.begin(), all.list.end(), pool));
+    cudaMemPoolDestroy(pool);
 }
 
 void* StreamPool::get(const Alloc& A, int device, size_t bytes, cudaStream_t s) {
@@ -78,6 +105,9 @@ void* StreamPool::get(const Alloc& A, int device, size_t bytes, cudaStream_t s) 
             pool = nullptr;
             return nullptr;
         }
+        Pools& all = Pools::all();
+        std::lock_guard<std::mutex> la(all.mu);
+        all.list.push_back(pool);
     }
     void* p = nullptr;
     if (cudaMallocFromPoolAsync(&p, bytes, pool, s) != cudaSuccess) {

@@ -40,7 +40,7 @@ struct DevBuf {
 // stream-ordered memory pool of its owner (a Hamiltonian, a batch), made on
 // first use and destroyed with the owner.  Calls on several streams or threads
 // each get memory of their own; up to KEEP bytes stay in the pool between
-// calls.  get returns null (the caller then does without) for a custom
+// calls, until an allocation of the library fails for want of them.  get returns null (the caller then does without) for a custom
 // allocator, on a capturing stream, and when the memory is not there.
 struct StreamPool {
     static constexpr uint64_t KEEP = 256ull << 20;
@@ -48,9 +48,8 @@ struct StreamPool {
     cudaMemPool_t pool = nullptr;
     void* get(const Alloc& A, int device, size_t bytes, cudaStream_t s);
     static void put(void* p, cudaStream_t s) { cudaFreeAsync(p, s); }
-    ~StreamPool() {
-        if (pool) cudaMemPoolDestroy(pool);
-    }
+    static bool trim();  // gives back what idles in every pool; false: there was no pool
+    ~StreamPool();
 };
 
 // ---------------------------------------------------------------- sublattice-coding tables (host)
