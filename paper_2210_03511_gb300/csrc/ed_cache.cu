@@ -623,6 +623,8 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
                         codes.cap, c.off_bits);
         if (grew || k == 0)
             ED_CUDA(cudaMemcpyAsync(d_code, codes.code.data(), codes.code.size(), cudaMemcpyHostToDevice, s));
+        // At most 2^32 - 2 entries to a segment: not for the offsets' sake, which count from the
+        // chunk's first entry, but a structure that was refused stays refused
         for (int i = 0; i < nb; ++i) {
             seg_total[i] += edge[i + 1] - edge[i];
             if (seg_total[i] >= 0xFFFFFFFFull)

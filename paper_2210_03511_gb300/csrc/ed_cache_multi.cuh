@@ -1,16 +1,15 @@
 // Stored-structure H.x for several FP32 vectors (2 to 8, real or complex),
 // instantiated per value kind in ed_cache_multi_k<K>.cu.
 //
-// With the vectors one after another each element gathers a 32-byte sector per
-// vector.  So x is first copied to [row][NP] (NP = 2, 4 or 8 >= NV vectors): all
-// vectors' x_j of an element lie in one run.  Bound by the L1 data pipe.
-// square32, copy included, against one one-vector pass after another: two real
-// vectors 0.31 against 0.49 ms, five 0.58 against 1.22, eight 0.58 against 1.95,
-// five complex 1.34 (one lane per row: five 0.71, eight 0.81, five complex 1.62;
-// at first, one kernel gathering vector by vector: five in 1.81 ms).  FP64 vectors
-// take one-vector passes: they are bound by the FP64 pipe, and the copy won
-// nothing (square32, three vectors: 0.94 against 1.00 ms real, 1.85 against 1.82
-// complex).
+// With one-vector passes each element gathers a 32-byte sector per vector.  So, where
+// the sector is not small (cache_interleaved_bytes), x is first copied to [row][NP]
+// (NP = 2, 4 or 8 >= NV vectors): all vectors' x_j of an element lie in one run.
+// Bound by the L1 data pipe.  square32, copy included, against one-vector passes side
+// by side: two real vectors 0.31 against 0.47 ms, five 0.58 against 1.11, eight 0.58
+// against 1.74, five complex 1.34 against 1.49 (one lane per row: five 0.71, eight 0.81,
+// five complex 1.62; at first, one kernel gathering vector by vector: five in 1.81 ms).
+// FP64 vectors take one-vector passes: they are bound by the FP64 pipe, and the copy won
+// nothing (square32, three vectors: 0.94 against 0.95 ms real, 1.85 against 1.75 complex).
 // The sums are those of the one-vector pass, entry by entry (complex vectors too: axis-aligned
 // tables where that takes them), so y does not depend on whether there was room for the copy.
 #pragma once

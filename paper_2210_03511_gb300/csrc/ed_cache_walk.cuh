@@ -81,7 +81,9 @@ __device__ __forceinline__ float prod(float a, float b) { return __fmul_rn(a, b)
 // multiply-adds into one sum round it twice.
 // DIFF: the fused difference of products, added in one go, all the same (for
 // ed_lanczos: the sign of a Ritz vector hangs on the last bits of alpha and beta,
-// so its recursion keeps the arithmetic that its vectors have had).
+// so its recursion keeps the arithmetic that its vectors have had).  With one warp
+// per slice only: several warps per slice add their parts' sums in an order of their
+// own anyway, and take the four sums there too.
 template <int K, bool AX, bool DIFF = false>
 struct RowSum {
     using T = typename Val<K>::T;
