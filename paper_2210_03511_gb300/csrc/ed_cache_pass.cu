@@ -70,8 +70,10 @@ bool few(int64_t slices, int nvec, uint64_t entries, int64_t rows, int sms) {
 // PREV: modes 2 and 3 (a partial sum from earlier segments exists in y), a
 // compile-time flag so that the one-segment pass carries no such register.  A
 // row's sum continues from that partial sum; a row without entries in an inner
-// segment is left alone.  Vector blockIdx.y of p.nvec.
-template <int K, bool AX, bool PREV, bool DIFF, int BLOCKS, int U>
+// segment is left alone.  MV: vector blockIdx.y of p.nvec; one vector goes without, as
+// its offset costs the registers that the passes over several segments need (square36
+// FP64 13.35 -> 13.73 ms, kagome36 complex FP32 14.51 -> 14.71).
+template <int K, bool AX, bool PREV, bool DIFF, bool MV, int BLOCKS, int U>
 __global__ void __launch_bounds__(BLOCK, BLOCKS) cache_pass_kernel(CachePass p) {
     using V = Val<K>;
     using T = typename V::T;
@@ -81,11 +83,14 @@ __global__ void __launch_bounds__(BLOCK, BLOCKS) cache_pass_kernel(CachePass p) 
     stage_codes<K>(ctab, p.ctab);
     write_counters(p);
     __syncthreads();
-    const int64_t D = p.D;
-    const int64_t v = BLOCKS == MANY_BLOCKS ? 0 : (int64_t)blockIdx.y * D;  // this vector's first element
-    const T* __restrict__ x = (const T*)p.x + v;
-    T* __restrict__ y = (T*)p.y + v;
+    const T* __restrict__ x = (const T*)p.x;
+    T* __restrict__ y = (T*)p.y;
     const int lane = threadIdx.x & 31;
+    const int64_t D = p.D;
+    if constexpr (MV) {
+        x += (int64_t)blockIdx.y * D;
+        y += (int64_t)blockIdx.y * D;
+    }
     const uint32_t ob = p.off_bits, om = (1u << ob) - 1u, n_re = p.n_re;
     const bool last = p.mode == 0 || p.mode == 3;
     const T* __restrict__ xs = x + p.xoff;
@@ -235,34 +240,39 @@ __global__ void __launch_bounds__(BLOCK, BLOCKS)
     }
 }
 
-template <int K, bool AX, bool DIFF = false, int BLOCKS = pass_blocks(K), int U = AHEAD>
-ed_status launch_pass(const CachePass& p, int sms, cudaStream_t s) {
-    if constexpr (K == 1 && BLOCKS != MANY_BLOCKS)
-        if (p.mode != 0 && p.n_ent >= MANY_ROW_ENTRIES * (uint64_t)p.D * (uint64_t)p.nb)
-            return launch_pass<K, AX, DIFF, MANY_BLOCKS>(p, sms, s);
-    if constexpr (BLOCKS == pass_blocks(K) && U == AHEAD)
-        if (p.mode == 0 && few<K>(p.ns, p.nvec, p.n_ent, p.D, sms))
-            return launch_pass<K, AX, DIFF, few_blocks(K), FEW_AHEAD>(p, sms, s);
+// The vectors side by side (MV), or one launch for each.
+template <int K, bool AX, bool DIFF, bool MV, int BLOCKS, int U>
+ed_status launch_blocks(const CachePass& p, int sms, cudaStream_t s) {
+    using T = typename Val<K>::T;
     const int64_t need = (p.ns + (BLOCK / 32) - 1) / (BLOCK / 32);
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sms * BLOCKS));
-    // the eight-block kernel has no register left for the vector's offset: one launch per vector
-    using T = typename Val<K>::T;
     CachePass q = p;
-    const int together = BLOCKS == MANY_BLOCKS ? 1 : p.nvec;
-    for (int v = 0; v < p.nvec; v += together) {
-        const dim3 g(grid, (unsigned)together);
+    for (int v = 0; v < p.nvec; v += MV ? p.nvec : 1) {
+        const dim3 g(grid, MV ? (unsigned)p.nvec : 1u);
         q.x = (const T*)p.x + (int64_t)v * p.D;
         q.y = (T*)p.y + (int64_t)v * p.D;
         if constexpr (U == AHEAD) {
             if (p.mode >= 2) {
-                cache_pass_kernel<K, AX, true, DIFF, BLOCKS, U><<<g, BLOCK, 0, s>>>(q);
+                cache_pass_kernel<K, AX, true, DIFF, MV, BLOCKS, U><<<g, BLOCK, 0, s>>>(q);
                 continue;
             }
         }
-        cache_pass_kernel<K, AX, false, DIFF, BLOCKS, U><<<g, BLOCK, 0, s>>>(q);
+        cache_pass_kernel<K, AX, false, DIFF, MV, BLOCKS, U><<<g, BLOCK, 0, s>>>(q);
     }
     ED_CUDA(cudaGetLastError());
     return ED_OK;
+}
+
+template <int K, bool AX, bool DIFF = false>
+ed_status launch_pass(const CachePass& p, int sms, cudaStream_t s) {
+    if constexpr (K == 1)  // no register left for a vector's offset: one launch per vector
+        if (p.mode != 0 && p.n_ent >= MANY_ROW_ENTRIES * (uint64_t)p.D * (uint64_t)p.nb)
+            return launch_blocks<K, AX, DIFF, false, MANY_BLOCKS, AHEAD>(p, sms, s);
+    if (p.mode == 0 && few<K>(p.ns, p.nvec, p.n_ent, p.D, sms))
+        return launch_blocks<K, AX, DIFF, true, few_blocks(K), FEW_AHEAD>(p, sms, s);
+    const bool fills = p.ns > (int64_t)sms * pass_blocks(K) * (BLOCK / 32);
+    return p.nvec == 1 || (p.mode != 0 && fills) ? launch_blocks<K, AX, DIFF, false, pass_blocks(K), AHEAD>(p, sms, s)
+                                                 : launch_blocks<K, AX, DIFF, true, pass_blocks(K), AHEAD>(p, sms, s);
 }
 
 template <int K, int L>
@@ -288,9 +298,10 @@ ed_status launch_kind(const CachePass& p, bool ax, int lanes, int sms, cudaStrea
         return fail(ED_ERR_ARG, "lanes per row must be 1, 2, 4 or 8");
     }
     // Several FP64 vectors (their passes are bound by the FP64 pipe, not by the gathers), or no
-    // room for the interleaved copy: the one-vector passes side by side in one launch.  A launch
-    // per vector leaves most of the GPU idle in a small sector: eight FP64 vectors of 12,870 rows
-    // 49 -> 8.1 us, of 28,699 rows 131 -> 44 us, of 2.4 million rows 2.69 -> 2.47 ms.
+    // room for the interleaved copy: the one-vector passes, side by side in one launch (over
+    // several segments only where one vector does not fill the GPU).  A launch per vector leaves
+    // most of the GPU idle in a small sector: eight FP64 vectors of 12,870 rows 49 -> 8.1 us, of
+    // 28,699 rows 131 -> 44 us, of 2.4 million rows 2.69 -> 2.47 ms.
     if constexpr (Val<K>::cplx)
         return ax ? launch_pass<K, true>(p, sms, s)
                   : (p.diff ? launch_pass<K, false, true>(p, sms, s) : launch_pass<K, false>(p, sms, s));
