@@ -299,11 +299,12 @@ void ed_hamiltonian_free(ed_hamiltonian* h);
  * y_i = sum_j conj(H_ji) x_j, valid because H is Hermitian).
  * Two to eight FP32 vectors on a stored structure (ed_hamiltonian_store) are
  * copied interleaved by row, unless the sector is small: stream-ordered device
- * scratch of up to 8 D elements, from a memory pool of the Hamiltonian and not
- * from its allocator.  A Hamiltonian with an allocator of the caller's, a
- * captured call and a full device do without it, with the same results.
+ * scratch of up to 8 D elements, from a memory pool of the device and not from
+ * the Hamiltonian's allocator.  A Hamiltonian with an allocator of the caller's,
+ * a captured call and a full device do without it, with the same results.
  * At most 256 MB stay in the pool between calls; they go when an allocation of
- * this library finds no memory and with the Hamiltonian.
+ * this library finds no memory, and with the last Hamiltonian or batch that
+ * took any.
  * Asynchronous on `stream`. */
 ed_status ed_apply(const ed_hamiltonian* h, ed_dtype dtype, const void* x, void* y, int32_t nvec, ed_stream stream);
 
@@ -548,7 +549,7 @@ ed_status ed_batch_rows(const ed_batch* batch, int64_t* row_off);
  * launch: every block takes a contiguous range of the batch's rows and stages
  * each sector's tables as it reaches its rows.  x, y: DEVICE, caller-owned.
  * With every sector's structure stored, two to eight FP32 vectors take scratch
- * of up to 8 elements per row from a pool of the batch, as in ed_apply.
+ * of up to 8 elements per row from the device's pool, as in ed_apply.
  * Asynchronous on `stream`. */
 ed_status ed_apply_batch(const ed_batch* batch, ed_dtype dtype, const void* x, void* y, int32_t nvec, ed_stream stream);
 

@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -58,30 +59,53 @@ void Alloc::put(void* p, size_t bytes, cudaStream_t s) const {
     else cudaFree(p);
 }
 
-// The pools that exist.  Never destroyed: owners may be freed at any time before exit.
+// The devices' pools and how many objects have taken memory from them.  Never destroyed:
+// objects may be freed at any time before exit.
 struct Pools {
     std::mutex mu;
-    std::vector<cudaMemPool_t> list;
+    std::map<int, cudaMemPool_t> of;
+    int owners = 0;
     static Pools& all() {
         static Pools* p = new Pools;
         return *p;
+    }
+    void trim() {
+        for (auto& p : of) cudaMemPoolTrimTo(p.second, 0);
+        cudaGetLastError();
+    }
+    cudaMemPool_t get(int device) {
+        auto it = of.find(device);
+        if (it != of.end()) return it->second;
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        cudaMemPool_t pool = nullptr;
+        uint64_t keep = StreamPool::KEEP;
+        int no = 0;  // a call never waits for another stream's memory
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+            cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no) != cudaSuccess) {
+            cudaGetLastError();
+            if (pool) cudaMemPoolDestroy(pool);
+            return nullptr;
+        }
+        of[device] = pool;
+        return pool;
     }
 };
 
 bool StreamPool::trim() {
     Pools& all = Pools::all();
     std::lock_guard<std::mutex> l(all.mu);
-    for (cudaMemPool_t p : all.list) cudaMemPoolTrimTo(p, 0);
-    cudaGetLastError();
-    return !all.list.empty();
+    all.trim();
+    return !all.of.empty();
 }
 
 StreamPool::~StreamPool() {
-    if (!pool) return;
     Pools& all = Pools::all();
     std::lock_guard<std::mutex> l(all.mu);
-    all.list.erase(std::find(all.list.begin(), all.list.end(), pool));
-    cudaMemPoolDestroy(pool);
+    if (used && --all.owners == 0) all.trim();
 }
 
 void* StreamPool::get(const Alloc& A, int device, size_t bytes, cudaStream_t s) {
@@ -91,23 +115,16 @@ void* StreamPool::get(const Alloc& A, int device, size_t bytes, cudaStream_t s) 
         cudaGetLastError();
         return nullptr;
     }
-    std::lock_guard<std::mutex> l(mu);
-    if (!pool) {
-        cudaMemPoolProps props{};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = device;
-        uint64_t keep = KEEP;
-        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
-            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaGetLastError();
-            if (pool) cudaMemPoolDestroy(pool);
-            pool = nullptr;
-            return nullptr;
-        }
+    cudaMemPool_t pool;
+    {
         Pools& all = Pools::all();
-        std::lock_guard<std::mutex> la(all.mu);
-        all.list.push_back(pool);
+        std::lock_guard<std::mutex> l(all.mu);
+        pool = all.get(device);
+        if (!pool) return nullptr;
+        if (!used) {
+            used = true;
+            ++all.owners;
+        }
     }
     void* p = nullptr;
     if (cudaMallocFromPoolAsync(&p, bytes, pool, s) != cudaSuccess) {

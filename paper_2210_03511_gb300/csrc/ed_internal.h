@@ -5,7 +5,6 @@
 #include <stdint.h>
 
 #include <string>
-#include <mutex>
 #include <vector>
 
 #include "ed.h"
@@ -36,20 +35,27 @@ struct DevBuf {
     size_t bytes = 0;
 };
 
-// Device scratch of calls that are asynchronous on their stream: a
-// stream-ordered memory pool of its owner (a Hamiltonian, a batch), made on
-// first use and destroyed with the owner.  Calls on several streams or threads
-// each get memory of their own; up to KEEP bytes stay in the pool between
-// calls, until an allocation of the library fails for want of them.  get returns null (the caller then does without) for a custom
-// allocator, on a capturing stream, and when the memory is not there.
-struct StreamPool {
+// Device scratch of calls that are asynchronous on their stream: one stream-ordered
+// memory pool per device, made on first use (making a pool and mapping its first memory
+// take 0.1 ms, which a pool per Hamiltonian paid on each one's first call).  Calls on
+// several streams or threads each get memory of their own, and none waits for another's.
+// Up to KEEP bytes idle in the pool between calls; they are given back when the last
+// Hamiltonian or batch that took any is freed, and when an allocation of the library fails
+// for want of them.
+class StreamPool {
+    bool used = false;  // counted among the pools' owners (guarded by their mutex)
+
+  public:
     static constexpr uint64_t KEEP = 256ull << 20;
-    std::mutex mu;
-    cudaMemPool_t pool = nullptr;
+    StreamPool() = default;
+    StreamPool(const StreamPool&) = delete;
+    StreamPool& operator=(const StreamPool&) = delete;
+    ~StreamPool();
+    // null (the caller then does without) for a custom allocator, on a capturing stream, and
+    // when the memory is not there
     void* get(const Alloc& A, int device, size_t bytes, cudaStream_t s);
     static void put(void* p, cudaStream_t s) { cudaFreeAsync(p, s); }
-    static bool trim();  // gives back what idles in every pool; false: there was no pool
-    ~StreamPool();
+    static bool trim();  // gives back what idles; false: there is no pool
 };
 
 // ---------------------------------------------------------------- sublattice-coding tables (host)

@@ -47,3 +47,36 @@ def test_idle_scratch_is_given_back(P):
     finally:
         del fill
         torch.cuda.empty_cache()
+
+
+def test_one_pool(P):
+    """A second Hamiltonian's call on a stream takes the scratch that idles there after the first
+    one's (another stream may take memory of its own); freeing both gives all of it back."""
+    import torch
+    p = C.square32()
+    b = P.Basis(p.sector)
+    hs = [P.Hamiltonian(b, p.terms) for _ in range(2)]
+    x = torch.randn((8, b.dim), dtype=torch.float32, device="cuda")
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    for h in hs:
+        h.store(P.ED_F32)
+        h.apply(x[0], y[0])
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    hs[0].apply(x, y)
+    torch.cuda.synchronize()
+    taken = torch.cuda.mem_get_info()[0]
+    assert taken < before
+    hs[1].apply(x, z)
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] >= taken
+    assert torch.equal(y, z)
+    z.zero_()
+    torch.cuda.synchronize()
+    hs[1].apply(x, z, stream=torch.cuda.Stream())
+    torch.cuda.synchronize()
+    assert torch.equal(y, z)
+    held = sum(h.store_info()["bytes"] for h in hs)
+    for h in hs:
+        h.close()
+    assert torch.cuda.mem_get_info()[0] >= before + held // 2
