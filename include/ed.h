@@ -337,7 +337,8 @@ ed_status ed_apply(const ed_hamiltonian* h, ed_dtype dtype, const void* x, void*
  * ED_ERR_ARG for more than 255 flip terms.  The build takes scratch from the
  * same allocator (8 bytes per flip term and row for a chunk of rows, up to
  * about 3 GB; less when the allocator has no room for that, down to a few per
- * cent of the structure), released on return.
+ * cent of the structure), released on return; without an allocator of the
+ * caller's, scratch of 1 to 16 MB comes from the device's pool (ed_apply).
  * Synchronous on `stream`.
  * A second call replaces the stored structure. */
 ed_status ed_hamiltonian_store(ed_hamiltonian* h, ed_dtype dtype, int32_t seg_log2, size_t max_bytes,

@@ -490,6 +490,12 @@ struct Codes {
     }
 };
 
+// Scratch of these sizes comes from the device's pool: an allocation of more than 1 MB takes
+// 0.13 ms to map and free, as much as the search of a small sector (kagome18 without rotations,
+// 8,110 rows: 0.44 -> 0.36 ms, triangular24 0.75 -> 0.65); smaller ones are cheap, and large
+// sectors do not notice.
+constexpr size_t POOLED_MIN = (size_t)1 << 20, POOLED_MAX = (size_t)16 << 20;
+
 // Builds the structure into h->cache, its chunks' scratch limited to about
 // `scratch` bytes.  On an error the parts stay in h->cache for cache_free;
 // smaller: the scratch of another try, where the memory had no room for this one's
@@ -511,9 +517,9 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
     const int64_t ns = c.ns, Dpad = ns * NSLICE;
     // chunk: a power of two of rows whose raw entries fit the scratch; the only chunk: all rows.
     // Column and key in one word where they fit (32-bit states; sectors of 64-bit states are large,
-    // and the choice cost their search 4 %, square36 219 -> 229 ms): an allocation that needs 2 MB
-    // of its own costs as much as the build of a small sector (chain16, 12,870 rows: 0.30 ms with
-    // two words, 0.16 with one; square32 7.0 -> 5.8 ms)
+    // and the choice cost their search 4 %, square36 219 -> 229 ms): half the scratch, which in a
+    // small sector then stays below what an allocation of its own takes (chain16, 12,870 rows:
+    // 0.30 -> 0.16 ms), and half its traffic (square32 7.0 -> 5.8 ms)
     auto width = [](uint64_t n) {
         int k = 1;
         while (((uint64_t)1 << k) < n) ++k;
@@ -550,7 +556,14 @@ static ed_status build_once(ed_hamiltonian* h, int bits, size_t max_bytes, size_
                  o_raw = part((size_t)std::max(h->n_flip, 1) * R * raw_bytes), o_tot1 = part((size_t)R),
                  o_tot = part((size_t)nb * Rsl * 4), o_abs = part(((size_t)nb * Rsl + 1) * 8),
                  o_tiles = part(scan_scratch_words((uint64_t)nb * Rsl) * 8);
-    uint8_t* scr = (uint8_t*)sc.get(at);
+    struct Pooled {
+        void* p;
+        cudaStream_t s;
+        ~Pooled() {
+            if (p) StreamPool::put(p, s);
+        }
+    } pooled{at > POOLED_MIN && at <= POOLED_MAX ? h->scratch.get(A, b->device, at, s) : nullptr, s};
+    uint8_t* scr = (uint8_t*)(pooled.p ? pooled.p : sc.get(at));
     uint16_t* d_hmap = (uint16_t*)(scr + o_hmap);
     uint16_t* d_chi = (uint16_t*)(scr + o_chi);
     unsigned long long* d_cnt = (unsigned long long*)(scr + o_cnt);

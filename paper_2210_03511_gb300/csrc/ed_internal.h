@@ -35,7 +35,8 @@ struct DevBuf {
     size_t bytes = 0;
 };
 
-// Device scratch of calls that are asynchronous on their stream: one stream-ordered
+// Device scratch of calls that are asynchronous on their stream (and small scratch of
+// structure builds): one stream-ordered
 // memory pool per device, made on first use (making a pool and mapping its first memory
 // take 0.1 ms, which a pool per Hamiltonian paid on each one's first call).  Calls on
 // several streams or threads each get memory of their own, and none waits for another's.
@@ -199,7 +200,7 @@ struct ed_hamiltonian {
     int tuned_blocks[4][2] = {};        // resident H.x blocks per SM by dtype, nvec == 1 / > 1 (0: default)
     bool sun = false;                   // SU(N) exchange model: applied through its stored structure only
     ed::HCache cache;                   // stored structure, when built (ed_hamiltonian_store)
-    mutable ed::StreamPool scratch;     // interleaved copies of several FP32 vectors (stored H.x)
+    mutable ed::StreamPool scratch;     // interleaved copies of several FP32 vectors (stored H.x), small builds
 };
 
 namespace ed {
